@@ -394,6 +394,16 @@ DevScene prepare(const cem_scene_desc& s, const cem_skeleton_desc& k) {
     }
     d.bslab_n[gi] = nb;
   }
+  // a projection on n changes by at most max |n_i| per metre of path (1 for
+  // the unit normals the descriptor asks for)
+  float nmax = 1.0f;
+  for (int gi = 0; gi < s.n_geoms; ++gi)
+    for (int si = 0; si < s.geom[gi].n_slabs; ++si)
+      for (int j = 0; j < 3; ++j) {
+        const float a = std::fabs(s.geom[gi].slab[si].n[j]);
+        nmax = a <= nmax ? nmax : a;
+      }
+  d.sep_scale = std::isfinite(nmax) ? 1.0f / nmax : 0.0f;
   for (int i = 0; i < CEM_MAX_D; ++i) d.theta_star[i] = s.theta_star[i];
   for (int i = 0; i < k.D * k.D; ++i) d.A[i] = s.A[i];
   if (s.kind == CEM_SCENE_PICKPLACE && s.base_controller == 1) {
