@@ -340,61 +340,79 @@ __device__ __noinline__ void planar_rollout(const DevScene& s, const float* __re
 }
 
 // --------------------------------------------------------------- pick-place
-// Minimum-overlap contact of an axis-aligned mover against static geometry g.
-// The mover's support along each slab normal is folded into the slab when
-// the scene is prepared (DevScene::oslab for the object cube, ::bslab for
-// the base footprint's slabs with n_z == 0), so a slab costs one projection
-// and two differences: overlap through the 'hi' side hi' - p.n, through the
-// 'lo' side p.n - lo'.  The smallest overlap (first on ties) gives the
-// outward normal and the depth; any separating slab means no contact, and
-// the gap along the first one found lowers `sep` (see kSkin below).
+// Overlap of an axis-aligned mover with slab i of static geometry g.  The
+// mover's support along each slab normal is folded into the slab when the
+// scene is prepared (DevScene::oslab for the object cube, ::bslab for the
+// base footprint's slabs with n_z == 0), so a slab costs one projection and
+// two differences: through the 'hi' side hi' - p.n, through the 'lo' side
+// p.n - lo'; `ov` is the smaller, n the outward normal of its side (as a
+// sign on the slab's axis).  Rounding pinned (no contraction choices left to
+// the compiler): every lane-group width evaluates a contact with the same
+// operations.
+struct Overlap {
+  float ov, nx, ny, nz;
+};
 template <bool PLANAR>
-__device__ __forceinline__ bool slab_contact(const DevScene& s, int g, float px, float py, float pz, float& nx,
-                                             float& ny, float& nz, float& depth, float& sep) {
+__device__ __forceinline__ Overlap slab_overlap(const DevScene& s, int g, int i, float px, float py, float pz) {
+  float4 sl;
+  float lo, hi, sp;
+  if (PLANAR) {
+    sl = *reinterpret_cast<const float4*>(s.bslab[g][i]);
+    lo = sl.z;
+    hi = sl.w;
+    sl.z = 0.0f;
+    sp = __fmaf_rn(sl.x, px, __fmul_rn(sl.y, py));
+  } else {
+    sl = *reinterpret_cast<const float4*>(s.oslab[g][i]);
+    lo = sl.w;
+    hi = s.oslab[g][i][4];
+    sp = __fmaf_rn(sl.x, px, __fmaf_rn(sl.y, py, __fmul_rn(sl.z, pz)));
+  }
+  const float ov_pos = __fsub_rn(hi, sp);
+  const float ov_neg = __fsub_rn(sp, lo);
+  const float sg = ov_pos <= ov_neg ? 1.0f : -1.0f;
+  return Overlap{fminf(ov_pos, ov_neg), sg * sl.x, sg * sl.y, sg * sl.z};
+}
+
+// Minimum-overlap contact against geometry g: the slab with the smallest
+// overlap (first on ties) gives the outward normal and the depth o.ov; a
+// negative or zero one separates the bodies.  ov2: the second smallest (1e30
+// if there is none); returns the slab's index (-1: the geometry has none).
+// Slabs are read in pairs, so that their shared-memory latencies overlap.
+template <bool PLANAR>
+__device__ __forceinline__ int least_overlap(const DevScene& s, int g, float px, float py, float pz, Overlap& o,
+                                             float& ov2) {
   g = CEM_DIDX(g, s.n_geoms, 6);
-  bool any = false;
-  float best = 0.0f;
   const int ns = PLANAR ? s.bslab_n[g] : s.geom_nslab[g];
-  for (int i = 0; i < ns; ++i) {
-    // rounding pinned (no contraction choices left to the compiler): every
-    // lane-group width evaluates a contact with the same operations
-    float n0, n1, n2, sp, lo, hi;
-    if (PLANAR) {
-      const float4 sl = *reinterpret_cast<const float4*>(s.bslab[g][i]);
-      n0 = sl.x;
-      n1 = sl.y;
-      n2 = 0.0f;
-      sp = __fmaf_rn(n0, px, __fmul_rn(n1, py));
-      lo = sl.z;
-      hi = sl.w;
+  static_assert(CEM_MAX_SLABS % 2 == 0, "slabs are read in pairs");
+  o.ov = ov2 = 1e30f;
+  int face = -1;
+  for (int i = 0; i < ns; i += 2) {
+    const Overlap u = slab_overlap<PLANAR>(s, g, i, px, py, pz);
+    Overlap v = slab_overlap<PLANAR>(s, g, i + 1, px, py, pz);
+    if (i + 1 >= ns) v.ov = 1e30f;
+    if (i == 0 || u.ov < o.ov) {
+      ov2 = o.ov;
+      o = u;
+      face = i;
     } else {
-      const float4 sl = *reinterpret_cast<const float4*>(s.oslab[g][i]);
-      n0 = sl.x;
-      n1 = sl.y;
-      n2 = sl.z;
-      sp = __fmaf_rn(n0, px, __fmaf_rn(n1, py, __fmul_rn(n2, pz)));
-      lo = sl.w;
-      hi = s.oslab[g][i][4];
+      ov2 = fminf(ov2, u.ov);
     }
-    const float ov_pos = __fsub_rn(hi, sp);
-    const float ov_neg = __fsub_rn(sp, lo);
-    const float ov = fminf(ov_pos, ov_neg);
-    if (ov_pos <= 0.0f || ov_neg <= 0.0f) {
-      sep = fminf(sep, fabsf(ov));
-      return false;
-    }
-    if (!any || ov < best) {
-      best = ov;
-      any = true;
-      const float sg = ov_pos <= ov_neg ? 1.0f : -1.0f;
-      nx = sg * n0;
-      ny = sg * n1;
-      nz = sg * n2;
+    if (v.ov < o.ov) {
+      ov2 = o.ov;
+      o = v;
+      face = i + 1;
+    } else {
+      ov2 = fminf(ov2, v.ov);
     }
   }
-  depth = best;
-  return any;
+  return face;
 }
+
+// Contact lists (see Reach).  A body left out of a list is at least kSkin away
+// along some world axis; a new list once the mover's path has grown by
+// kRebuild keeps it at least 1 cm clear (far above FP32 rounding).
+constexpr float kSkin = 0.15f, kRebuild = 0.14f, kTight = 0.02f;
 
 // A group of G consecutive lanes (G = 1, 8 or 32) sharing one rollout: every
 // lane holds the same state and runs the same serial dynamics, the group
@@ -423,30 +441,15 @@ __device__ __forceinline__ int nth_bit(uint32_t m, int k) {
   return __ffs(m) - 1;
 }
 
-// Penalty force on the base footprint from geometry g: F_n = max(0, k depth -
-// c v_n) along the minimum-overlap normal, returned as (cx, cy) = F_n n.
-__device__ __forceinline__ bool base_force(const DevScene& s, int g, float bx, float by, float bvx, float bvy,
-                                           float kc, float cc, float& cx, float& cy, float& sep) {
-  float nx, ny, nz, dep;
-  if (!slab_contact<true>(s, g, bx, by, 0.0f, nx, ny, nz, dep, sep)) return false;
-  sep = 0.0f;
-  const float vn = __fmaf_rn(bvx, nx, __fmul_rn(bvy, ny));
-  const float Fn = fmaxf(0.0f, __fsub_rn(__fmul_rn(kc, dep), __fmul_rn(cc, vn)));
-  cx = __fmul_rn(Fn, nx);
-  cy = __fmul_rn(Fn, ny);
-  return true;
+// Penalty force of one contact: F_n = max(0, k depth - c v_n) along the
+// outward normal n, v_n the velocity along it.
+__device__ __forceinline__ float base_force(const Overlap& o, float bvx, float bvy, float kc, float cc) {
+  const float vn = __fmaf_rn(bvx, o.nx, __fmul_rn(bvy, o.ny));
+  return fmaxf(0.0f, __fsub_rn(__fmul_rn(kc, o.ov), __fmul_rn(cc, vn)));
 }
-
-// Normal and F_n of the object against geometry g (false: no overlap).
-__device__ __forceinline__ bool obj_force(const DevScene& s, int g, float px, float py, float pz, float vx, float vy,
-                                          float vz, float kc, float cc, float& nx, float& ny, float& nz, float& Fn,
-                                          float& sep) {
-  float dep;
-  if (!slab_contact<false>(s, g, px, py, pz, nx, ny, nz, dep, sep)) return false;
-  sep = 0.0f;
-  const float vn = __fmaf_rn(vx, nx, __fmaf_rn(vy, ny, __fmul_rn(vz, nz)));
-  Fn = fmaxf(0.0f, __fsub_rn(__fmul_rn(kc, dep), __fmul_rn(cc, vn)));
-  return true;
+__device__ __forceinline__ float obj_force(const Overlap& o, float vx, float vy, float vz, float kc, float cc) {
+  const float vn = __fmaf_rn(vx, o.nx, __fmaf_rn(vy, o.ny, __fmul_rn(vz, o.nz)));
+  return fmaxf(0.0f, __fsub_rn(__fmul_rn(kc, o.ov), __fmul_rn(cc, vn)));
 }
 
 // Jacobi friction impulse of one of nc object contacts (normal n, force Fn)
@@ -481,10 +484,12 @@ __device__ __forceinline__ bool obj_friction(const ObjPhys& op, float nx, float 
 // that gap stays positive, so the geometry is still separated and its
 // contact test would return no contact.  PLANAR: base footprint (x, y only).
 // A lane group splits the geometries (lane r tests g = r, r + G, ...) and
-// ORs the bits.
+// ORs the bits.  Out of line (rare): the step loop's hot code stays together.
 template <bool PLANAR, int G>
-__device__ __forceinline__ uint32_t near_list(const DevScene& s, int n_geoms, float px, float py, float pz, float hx,
-                                              float hy, float hz, float skin, const Group<G>& grp) {
+__device__ __noinline__ uint32_t near_list(const DevScene& s, float px, float py, float pz) {
+  const Group<G> grp;
+  const int n_geoms = s.n_geoms;
+  const float hx = PLANAR ? s.bhx : s.oh, hy = PLANAR ? s.bhy : s.oh, hz = s.oh, skin = kSkin;
   uint32_t m = 0;
   const int flag = PLANAR ? 1 : 2;
   for (int g = grp.rank; g < n_geoms; g += G) {
@@ -513,52 +518,175 @@ __device__ __forceinline__ uint32_t near_list(const DevScene& s, int n_geoms, fl
   return grp.any_bits(m);
 }
 
-// Sum of the base's contact forces over the neighbour list `nbr`, added to
-// (fx, fy) in ascending geometry order.  G > 1: the k-th neighbour belongs to
-// lane k % G, which evaluates it; the sum then takes each contacting
-// geometry's force from its owner lane, in the same order and with the same
-// roundings as one lane alone.
+// What a contact query learns of the bodies it tested: those within kTight
+// (`near`) and their smallest gap (0: a contact), the smallest gap of the
+// others, and the slab (8 g + i + 1) of the smallest overlap of a near body
+// with what the next slab's overlap is beyond it.
+struct Gaps {
+  uint32_t near = 0u, face = 0u;
+  float near_gap = 1e30f, far_gap = 1e30f, lead = 1e30f;
+  __device__ __forceinline__ void take(int g, int face_i, const Overlap& o, float ov2) {
+    if (face_i < 0) return;
+    const float gap = fmaxf(-o.ov, 0.0f);
+    if (gap <= kTight) {
+      near |= 1u << g;
+      near_gap = fminf(near_gap, fabsf(gap));
+      face = (uint32_t)(8 * g + face_i + 1);
+      lead = ov2 - o.ov;
+    } else {
+      far_gap = fminf(far_gap, gap);
+    }
+  }
+  template <int G>
+  __device__ __forceinline__ void combine(const Group<G>& grp) {  // (face and lead count for a single near body only)
+    near = grp.any_bits(near);
+    near_gap = grp.least(near_gap);
+    far_gap = grp.least(far_gap);
+    face = grp.any_bits(face);
+    lead = grp.least(lead);
+  }
+};
+
+// Contact queries of one mover.  `list`: the bodies within kSkin along every
+// world axis when the list was built; `tight`: those of them that the last
+// full query found within kTight; `face`: the slab (8 g + i) of the smallest
+// overlap, where only one body is tight.  `path` is the length of the mover's
+// way so far (|dx| + |dy| (+ |dz|) per step, rounded up), the others are the
+// lengths at which the next query is due, the next full one, and the next
+// list.
+//
+// A full query tells how far the mover may go before another body can come
+// into contact, and before another slab of a single tight body can have the
+// smallest overlap.  Until then that one slab decides: the body touches if
+// and only if this overlap is positive, and its normal and depth are the
+// contact's.  So between full queries (`rest`) a query tests one slab, or the
+// tight bodies if there are several, and none at all (`next`) while they are
+// clear too.  (A position that is not a number makes `path` none and ends
+// the queries: such a contact carries no force.)
+struct Reach {
+  float path = 0.0f, next = 0.0f, rest = 0.0f, skin = 0.0f;
+  uint32_t list = 0u, tight = 0u;
+  int face = -1;
+  __device__ __forceinline__ bool due() const { return path >= next; }
+  __device__ __forceinline__ bool full() const { return path >= rest; }
+  __device__ __forceinline__ bool stale() const { return path >= skin; }
+  __device__ __forceinline__ void forget() { next = rest = skin = path; }
+  __device__ __forceinline__ void rebuilt(uint32_t near_bodies) {
+    list = near_bodies;
+    next = rest = path;
+    skin = __fadd_rd(path, kRebuild);
+  }
+  // path that may pass with a gap: less 0.1 mm and a few ulps of the
+  // projections (positions of L1 size p1), scaled by the scene's largest
+  // normal component (sep_scale; 1 for unit normals)
+  __device__ __forceinline__ float until(const DevScene& s, float gap, float p1) const {
+    return __fadd_rd(path, fmaxf((gap - 1e-4f) * s.sep_scale - 4e-6f * p1, 0.0f));
+  }
+  __device__ __forceinline__ void queried_all(const DevScene& s, const Gaps& q, float p1) {
+    tight = q.near;
+    rest = fminf(until(s, q.far_gap, p1), skin);
+    // both overlaps change by up to the path, so half their difference is sure
+    const float same_face = fminf(until(s, 0.5f * q.lead, p1), rest);
+    face = -1;
+    if (__popc(tight) == 1 && q.lead > 4e-3f) {
+      face = (int)q.face - 1;
+      rest = same_face;
+    }
+    next = fminf(until(s, q.near_gap, p1), rest);
+  }
+  __device__ __forceinline__ void queried(const DevScene& s, float gap, float p1) { next = fminf(until(s, gap, p1), rest); }
+  // the bodies that a due query tests one by one (none where `face` decides)
+  __device__ __forceinline__ uint32_t bodies(bool all) const { return all ? list : face >= 0 ? 0u : tight; }
+};
+
+// The base's contacts with the bodies `nbr`, tested one by one: their forces
+// are added to (fx, fy) in ascending geometry order.  G > 1: the k-th body
+// belongs to lane k % G, which evaluates it; the sum then takes each
+// contacting geometry's force from its owner lane, in the same order and with
+// the same roundings as one lane alone.  Out of line, as near_list.
+struct BaseQuery {
+  float fx, fy;
+  Gaps gaps;
+};
 template <int G>
-__device__ __forceinline__ void base_contacts(const DevScene& s, uint32_t nbr, float bx, float by, float bvx,
-                                              float bvy, float kc, float cc, const Group<G>& grp, float& fx,
-                                              float& fy, float& sep) {
+__device__ __noinline__ BaseQuery base_bodies(const DevScene& s, uint32_t nbr, float bx, float by, float bvx, float bvy,
+                                              float fx, float fy) {
+  const Group<G> grp;
+  const float kc = s.k_contact, cc = s.c_contact;
+  Gaps gaps;
+  Overlap o;
+  float ov2;
   if (G == 1) {
     for (uint32_t m = nbr; m; m &= m - 1u) {
-      float cx, cy;
-      if (base_force(s, __ffs(m) - 1, bx, by, bvx, bvy, kc, cc, cx, cy, sep)) {
-        fx = __fadd_rn(fx, cx);
-        fy = __fadd_rn(fy, cy);
+      const int g = __ffs(m) - 1;
+      const int face = least_overlap<true>(s, g, bx, by, 0.0f, o, ov2);
+      if (face >= 0 && o.ov > 0.0f) {
+        const float Fn = base_force(o, bvx, bvy, kc, cc);
+        fx = __fadd_rn(fx, __fmul_rn(Fn, o.nx));
+        fy = __fadd_rn(fy, __fmul_rn(Fn, o.ny));
+      }
+      gaps.take(g, face, o, ov2);
+    }
+  } else {
+    constexpr int SL = (CEM_MAX_GEOMS + G - 1) / G;
+    float cx[SL], cy[SL];
+    uint32_t hit = 0;
+    const int nn = __popc(nbr);
+#pragma unroll
+    for (int j = 0; j < SL; ++j) {
+      cx[j] = cy[j] = 0.0f;
+      const int k = grp.rank + j * G;
+      if (k < nn) {
+        const int g = nth_bit(nbr, k);
+        const int face = least_overlap<true>(s, g, bx, by, 0.0f, o, ov2);
+        if (face >= 0 && o.ov > 0.0f) {
+          const float Fn = base_force(o, bvx, bvy, kc, cc);
+          cx[j] = __fmul_rn(Fn, o.nx);
+          cy[j] = __fmul_rn(Fn, o.ny);
+          hit |= 1u << g;
+        }
+        gaps.take(g, face, o, ov2);
       }
     }
-    return;
-  }
-  constexpr int SL = (CEM_MAX_GEOMS + G - 1) / G;
-  float cx[SL], cy[SL];
-  uint32_t hit = 0;
-  const int nn = __popc(nbr);
+    gaps.combine(grp);
+    for (uint32_t m = grp.any_bits(hit); m; m &= m - 1u) {
+      const int g = __ffs(m) - 1;
+      const int k = __popc(nbr & ((1u << g) - 1u));
+      const int j = k / G, src = k & (G - 1);
+      float vx = cx[0], vy = cy[0];
 #pragma unroll
-  for (int j = 0; j < SL; ++j) {
-    cx[j] = cy[j] = 0.0f;
-    const int k = grp.rank + j * G;
-    if (k < nn) {
-      const int g = nth_bit(nbr, k);
-      if (base_force(s, g, bx, by, bvx, bvy, kc, cc, cx[j], cy[j], sep)) hit |= 1u << g;
+      for (int i = 1; i < SL; ++i)
+        if (j == i) {
+          vx = cx[i];
+          vy = cy[i];
+        }
+      fx = __fadd_rn(fx, grp.from(vx, src));
+      fy = __fadd_rn(fy, grp.from(vy, src));
     }
   }
-  sep = grp.least(sep);
-  for (uint32_t m = grp.any_bits(hit); m; m &= m - 1u) {
-    const int g = __ffs(m) - 1;
-    const int k = __popc(nbr & ((1u << g) - 1u));
-    const int j = k / G, src = k & (G - 1);
-    float vx = cx[0], vy = cy[0];
-#pragma unroll
-    for (int i = 1; i < SL; ++i)
-      if (j == i) {
-        vx = cx[i];
-        vy = cy[i];
-      }
-    fx = __fadd_rn(fx, grp.from(vx, src));
-    fy = __fadd_rn(fy, grp.from(vy, src));
+  return BaseQuery{fx, fy, gaps};
+}
+
+// One due query of the base's contacts (`all`: of the whole list), their
+// forces added to (fx, fy).
+template <int G>
+__device__ __forceinline__ void base_contacts(const DevScene& s, Reach& r, bool all, float bx, float by, float bvx,
+                                              float bvy, float kc, float cc, float& fx, float& fy) {
+  const float p1 = fabsf(bx) + fabsf(by);
+  if (!all && r.face >= 0) {
+    const Overlap o = slab_overlap<true>(s, CEM_DIDX(r.face >> 3, s.n_geoms, 6), r.face & 7, bx, by, 0.0f);
+    if (o.ov > 0.0f) {
+      const float Fn = base_force(o, bvx, bvy, kc, cc);
+      fx = __fadd_rn(fx, __fmul_rn(Fn, o.nx));
+      fy = __fadd_rn(fy, __fmul_rn(Fn, o.ny));
+    }
+    r.queried(s, fmaxf(-o.ov, 0.0f), p1);
+  } else {
+    const BaseQuery q = base_bodies<G>(s, r.bodies(all), bx, by, bvx, bvy, fx, fy);
+    fx = q.fx;
+    fy = q.fy;
+    if (all) r.queried_all(s, q.gaps, p1);
+    else r.queried(s, fminf(q.gaps.near_gap, q.gaps.far_gap), p1);
   }
 }
 
@@ -567,18 +695,24 @@ __device__ __forceinline__ float contact_share(int nc) {
   return nc == 1 ? 1.0f : nc == 2 ? 0.5f : __frcp_rn((float)nc);
 }
 
-// One object step against the static geometry in `nbr` (not attached):
-// penalty forces from the pre-step state, the trial velocity with gravity,
-// then one Jacobi friction impulse per contact from that trial velocity,
-// each summed in ascending geometry order.  Updates the velocity only.
+// One step of the free object's velocity against the bodies `nbr`, tested one
+// by one: penalty forces from the pre-step state, the trial velocity with
+// gravity, then one Jacobi friction impulse per contact from that trial
+// velocity, each summed in ascending geometry order.  Out of line, as
+// near_list.
+struct ObjQuery {
+  float vx, vy, vz;
+  Gaps gaps;
+};
 template <int G>
-__device__ __forceinline__ void object_contacts(const DevScene& s, const ObjPhys& op, uint32_t nbr, float ox,
-                                                float oy, float oz,
-                                                float& ovx, float& ovy, float& ovz, float kc, float cc,
-                                                const Group<G>& grp, float& sep) {
-  const float pvx = ovx, pvy = ovy, pvz = ovz;
+__device__ __noinline__ ObjQuery object_bodies(const DevScene& s, const ObjPhys op, uint32_t nbr, float ox, float oy,
+                                               float oz, float pvx, float pvy, float pvz) {
+  const Group<G> grp;
+  const float kc = s.k_contact, cc = s.c_contact;
   float fsx = 0.f, fsy = 0.f, fsz = 0.f;
   float jx = 0.f, jy = 0.f, jz = 0.f;
+  float ovx, ovy, ovz;
+  Gaps gaps;
   if (G == 1) {
     // the first two contacts (in ascending geometry order) are kept for the
     // friction pass; a third or later one is evaluated again there
@@ -587,18 +721,22 @@ __device__ __forceinline__ void object_contacts(const DevScene& s, const ObjPhys
     float n0x = 0.f, n0y = 0.f, n0z = 0.f, F0 = 0.f, n1x = 0.f, n1y = 0.f, n1z = 0.f, F1 = 0.f;
     for (uint32_t m = nbr; m; m &= m - 1u) {
       const int g = __ffs(m) - 1;
-      float nx, ny, nz, Fn;
-      if (obj_force(s, g, ox, oy, oz, pvx, pvy, pvz, kc, cc, nx, ny, nz, Fn, sep) && Fn > 0.0f) {
+      Overlap o;
+      float ov2;
+      const int face = least_overlap<false>(s, g, ox, oy, oz, o, ov2);
+      gaps.take(g, face, o, ov2);
+      const float Fn = face >= 0 && o.ov > 0.0f ? obj_force(o, pvx, pvy, pvz, kc, cc) : 0.0f;
+      if (Fn > 0.0f) {
         if (nc == 0) {
-          n0x = nx; n0y = ny; n0z = nz; F0 = Fn;
+          n0x = o.nx; n0y = o.ny; n0z = o.nz; F0 = Fn;
         } else if (nc == 1) {
-          n1x = nx; n1y = ny; n1z = nz; F1 = Fn;
+          n1x = o.nx; n1y = o.ny; n1z = o.nz; F1 = Fn;
         }
         cm |= 1u << g;
         ++nc;
-        fsx = __fadd_rn(fsx, __fmul_rn(Fn, nx));
-        fsy = __fadd_rn(fsy, __fmul_rn(Fn, ny));
-        fsz = __fadd_rn(fsz, __fmul_rn(Fn, nz));
+        fsx = __fadd_rn(fsx, __fmul_rn(Fn, o.nx));
+        fsy = __fadd_rn(fsy, __fmul_rn(Fn, o.ny));
+        fsz = __fadd_rn(fsz, __fmul_rn(Fn, o.nz));
       }
     }
     ovx = __fmaf_rn(op.dt_mo, fsx, pvx);
@@ -623,9 +761,11 @@ __device__ __forceinline__ void object_contacts(const DevScene& s, const ObjPhys
       rest &= rest - 1u;
       for (uint32_t m = rest; m; m &= m - 1u) {
         const int g = __ffs(m) - 1;
-        float nx, ny, nz, Fn;
-        obj_force(s, g, ox, oy, oz, pvx, pvy, pvz, kc, cc, nx, ny, nz, Fn, sep);
-        if (obj_friction(op, nx, ny, nz, Fn, ovx, ovy, ovz, inv_nc, cx, cy, cz)) {
+        Overlap o;
+        float ov2;
+        least_overlap<false>(s, g, ox, oy, oz, o, ov2);
+        if (obj_friction(op, o.nx, o.ny, o.nz, obj_force(o, pvx, pvy, pvz, kc, cc), ovx, ovy, ovz, inv_nc, cx, cy,
+                         cz)) {
           jx = __fsub_rn(jx, cx);
           jy = __fsub_rn(jy, cy);
           jz = __fsub_rn(jz, cz);
@@ -634,20 +774,25 @@ __device__ __forceinline__ void object_contacts(const DevScene& s, const ObjPhys
     }
   } else {
     constexpr int SL = (CEM_MAX_GEOMS + G - 1) / G;
-    float nx[SL], ny[SL], nz[SL], Fn[SL];
+    Overlap o[SL];
+    float Fn[SL];
     uint32_t hit = 0;
     const int nn = __popc(nbr);
 #pragma unroll
     for (int j = 0; j < SL; ++j) {
-      nx[j] = ny[j] = nz[j] = Fn[j] = 0.0f;
+      o[j] = Overlap{0.0f, 0.0f, 0.0f, 0.0f};
+      Fn[j] = 0.0f;
       const int k = grp.rank + j * G;
       if (k < nn) {
         const int g = nth_bit(nbr, k);
-        if (obj_force(s, g, ox, oy, oz, pvx, pvy, pvz, kc, cc, nx[j], ny[j], nz[j], Fn[j], sep) && Fn[j] > 0.0f)
-          hit |= 1u << g;
+        float ov2;
+        const int face = least_overlap<false>(s, g, ox, oy, oz, o[j], ov2);
+        gaps.take(g, face, o[j], ov2);
+        if (face >= 0 && o[j].ov > 0.0f) Fn[j] = obj_force(o[j], pvx, pvy, pvz, kc, cc);
+        if (Fn[j] > 0.0f) hit |= 1u << g;
       }
     }
-    sep = grp.least(sep);
+    gaps.combine(grp);
     const uint32_t cm = grp.any_bits(hit);
     const int nc = __popc(cm);
     const float inv_nc = contact_share(nc);
@@ -660,9 +805,9 @@ __device__ __forceinline__ void object_contacts(const DevScene& s, const ObjPhys
 #pragma unroll
       for (int i = 0; i < SL; ++i)
         if (j == i) {
-          a = __fmul_rn(Fn[i], nx[i]);
-          b = __fmul_rn(Fn[i], ny[i]);
-          c = __fmul_rn(Fn[i], nz[i]);
+          a = __fmul_rn(Fn[i], o[i].nx);
+          b = __fmul_rn(Fn[i], o[i].ny);
+          c = __fmul_rn(Fn[i], o[i].nz);
         }
       fsx = __fadd_rn(fsx, grp.from(a, src));
       fsy = __fadd_rn(fsy, grp.from(b, src));
@@ -680,7 +825,8 @@ __device__ __forceinline__ void object_contacts(const DevScene& s, const ObjPhys
       const int k = grp.rank + j * G;
       if (k < nn) {
         const int g = nth_bit(nbr, k);
-        if (((cm >> g) & 1u) && obj_friction(op, nx[j], ny[j], nz[j], Fn[j], ovx, ovy, ovz, inv_nc, fx[j], fy[j], fz[j]))
+        if (((cm >> g) & 1u) &&
+            obj_friction(op, o[j].nx, o[j].ny, o[j].nz, Fn[j], ovx, ovy, ovz, inv_nc, fx[j], fy[j], fz[j]))
           fr |= 1u << g;
       }
     }
@@ -701,10 +847,71 @@ __device__ __forceinline__ void object_contacts(const DevScene& s, const ObjPhys
       jz = __fsub_rn(jz, grp.from(c, src));
     }
   }
-  ovx = __fadd_rn(ovx, jx);
-  ovy = __fadd_rn(ovy, jy);
-  ovz = __fadd_rn(ovz, jz);
+  return ObjQuery{__fadd_rn(ovx, jx), __fadd_rn(ovy, jy), __fadd_rn(ovz, jz), gaps};
 }
+
+// One step of the free object's velocity (`due`: its contacts are queried,
+// `all`: those with the whole list).  Nothing or one slab to test is done
+// here, with object_bodies' arithmetic for no or one contact.
+template <int G>
+__device__ __forceinline__ void object_contacts(const DevScene& s, const ObjPhys& op, Reach& r, bool due, bool all,
+                                                float ox, float oy, float oz, float& ovx, float& ovy, float& ovz,
+                                                float kc, float cc) {
+  const float p1 = fabsf(ox) + fabsf(oy) + fabsf(oz);
+  if (due && (all || r.face < 0)) {
+    const ObjQuery q = object_bodies<G>(s, op, r.bodies(all), ox, oy, oz, ovx, ovy, ovz);
+    ovx = q.vx;
+    ovy = q.vy;
+    ovz = q.vz;
+    if (all) r.queried_all(s, q.gaps, p1);
+    else r.queried(s, fminf(q.gaps.near_gap, q.gaps.far_gap), p1);
+    return;
+  }
+  float Fn = 0.0f;
+  Overlap o{0.0f, 0.0f, 0.0f, 0.0f};
+  if (due) {
+    o = slab_overlap<false>(s, CEM_DIDX(r.face >> 3, s.n_geoms, 6), r.face & 7, ox, oy, oz);
+    if (o.ov > 0.0f) Fn = obj_force(o, ovx, ovy, ovz, kc, cc);
+    r.queried(s, fmaxf(-o.ov, 0.0f), p1);
+  }
+  ovx = __fmaf_rn(op.dt_mo, __fmul_rn(Fn, o.nx), ovx);
+  ovy = __fmaf_rn(op.dt_mo, __fmul_rn(Fn, o.ny), ovy);
+  ovz = __fsub_rn(__fmaf_rn(op.dt_mo, __fmul_rn(Fn, o.nz), ovz), __fmul_rn(s.g, s.dt));
+  if (Fn > 0.0f) {
+    float cx, cy, cz;
+    if (obj_friction(op, o.nx, o.ny, o.nz, Fn, ovx, ovy, ovz, 1.0f, cx, cy, cz)) {
+      ovx = __fsub_rn(ovx, cx);
+      ovy = __fsub_rn(ovy, cy);
+      ovz = __fsub_rn(ovz, cz);
+    }
+  }
+}
+
+#ifdef CEM_DEBUG
+// The step's contacts once more from every body, without lists or budgets: a
+// left-out query that would have found something is recorded (codes 10, 11).
+__device__ __noinline__ void check_base(const DevScene& s, float bx, float by, float bvx, float bvy, float kc, float cc,
+                                        float fx, float fy, float got_x, float got_y) {
+  for (int g = 0; g < s.n_geoms; ++g) {
+    Overlap o;
+    float ov2;
+    if (!(s.geom_flags[g] & 1) || least_overlap<true>(s, g, bx, by, 0.0f, o, ov2) < 0 || !(o.ov > 0.0f)) continue;
+    const float Fn = base_force(o, bvx, bvy, kc, cc);
+    fx = __fadd_rn(fx, __fmul_rn(Fn, o.nx));
+    fy = __fadd_rn(fy, __fmul_rn(Fn, o.ny));
+  }
+  if (fx < got_x || fx > got_x || fy < got_y || fy > got_y) (void)CEM_DIDX(1, 1, 10);
+}
+template <int G>
+__device__ __noinline__ void check_object(const DevScene& s, const ObjPhys op, float ox, float oy, float oz, float vx,
+                                          float vy, float vz, float got_x, float got_y, float got_z) {
+  uint32_t every = 0;
+  for (int g = 0; g < s.n_geoms; ++g)
+    if (s.geom_flags[g] & 2) every |= 1u << g;
+  const ObjQuery q = object_bodies<G>(s, op, every, ox, oy, oz, vx, vy, vz);
+  if (q.vx != got_x || q.vy != got_y || q.vz != got_z) (void)CEM_DIDX(1, 1, 11);
+}
+#endif
 
 // Analytic inverse kinematics of the 2-link arm in its vertical plane
 // (elbow up), returning the plane's azimuth as (cos, sin) = (dx, dy) / |d|
@@ -794,19 +1001,17 @@ __device__ __forceinline__ void arm_ee_velocity(const DevScene& s, float q1, flo
   vy = bvy + dr * sb;
 }
 
-// The path a mover may go before its next contact query, from the smallest
-// gap `sep` the last one found (0: a contact; positions of L1 size p1): less
-// 0.1 mm and a few ulps of the projections, scaled by the scene's largest
-// normal component (sep_scale; 1 for unit normals), and no further than the
-// list's own budget (clear + gap before the call).
-__device__ __forceinline__ void take_budget(const DevScene& s, float sep, float p1, float& clear, float& gap) {
-  const float left = fmaxf(__fadd_rd(clear, gap), 0.0f);
-  const float c = fminf((sep - 1e-4f) * s.sep_scale - 4e-6f * p1, left);
-  clear = c > 0.0f ? c : 0.0f;
-  gap = __fadd_rd(left, -clear);
+// kp e - kd v.  The step's arithmetic is written out with its roundings (which
+// products are fused), so that every instantiation and any arrangement of the
+// code around it simulates the same trajectory bit for bit.
+__device__ __forceinline__ float pd_law(float kp, float e, float kd, float v) {
+  return __fmaf_rn(kp, e, -__fmul_rn(kd, v));
+}
+__device__ __forceinline__ float norm2(float x, float y, float z) {
+  return __fmaf_rn(z, z, __fmaf_rn(x, x, __fmul_rn(y, y)));
 }
 
-constexpr int kQuietEvery = 8;  // steps between the looks for lanes at rest (a power of two)
+constexpr int kQuietEvery = 8;  // steps between the looks for lanes at rest (a power of two, 4 or more)
 
 // ASTAR = false compiles the A* base controller out (its waypoint arrays,
 // planning calls and integral state): a scene with the PD base takes that
@@ -816,11 +1021,11 @@ template <int G, bool TRACE, bool ASTAR>
 __device__ __noinline__ void pickplace_rollout(const DevScene& s, const float* __restrict__ row, int T, float smu,
                                                float sm, float& J_out, int& cls_out, float* tr) {
   const Group<G> grp;
-  const float dt = s.dt, h = s.oh, eps2 = s.eps * s.eps;
+  const float dt = s.dt;
   const float mb = s.mb, dt_mb = s.dt_mb, bcap = s.base_cap * smu, bcap2 = bcap * bcap;
   const ObjPhys op{s.obj_cap * smu, s.mo * sm, s.dt_mo / sm, 1.0f / (s.mo * sm)};
   const float kc = s.k_contact, cc = s.c_contact, akp = s.arm_kp, akd = s.arm_kd;
-  const int n_geoms = s.n_geoms;
+  const int L = s.n_act;
   float bx = s.base_start[0], by = s.base_start[1], bvx = s.base_v0[0], bvy = s.base_v0[1];
   float q1 = s.arm_home[0], q2 = s.arm_home[1], dq1 = 0.f, dq2 = 0.f, beta = 0.f;
   float cbeta = 1.0f, sbeta = 0.0f;
@@ -829,76 +1034,83 @@ __device__ __noinline__ void pickplace_rollout(const DevScene& s, const float* _
   float ovx = s.obj_v0[0], ovy = s.obj_v0[1], ovz = s.obj_v0[2];
   bool attached = false;
   float offx = 0.f, offy = 0.f, offz = 0.f;
-  float fk_r, fk_z;
-  arm_reach(s, q1, q2, fk_r, fk_z);
-  float ex = bx + fk_r * cbeta, ey = by + fk_r * sbeta, ez = fk_z;
-  const int L = s.n_act;
-  int a = 0, loaded = -1;
-  float gx = bx, gy = by, kp = 0.f, kd = 0.f;
-  float mgx = bx, mgy = by, mkp = 0.f, mkd = 0.f;
-  float rx = 0.f, ry = 0.f, caz = 1.f, saz = 0.f, hgrip = 0.f, ptx = 0.f, pty = 0.f, ptz = 0.f;
+  float ex, ey, ez;
+  {
+    float r, z;
+    arm_reach(s, q1, q2, r, z);
+    ex = __fmaf_rn(r, cbeta, bx);
+    ey = __fmaf_rn(r, sbeta, by);
+    ez = z;
+  }
+  // The action in progress: its kind, the base's goal and gains, the point
+  // (wx, wy, wz) that the base (a moveTo, wz = 0) or the end effector is to
+  // reach and the squared tolerance (negative: cannot succeed, or no action
+  // is left).  Set when the action starts; only a grasp, which aims at the
+  // object, renews its point.
+  int a = 0, kind = CEM_ACT_MOVE, last_move = -1;
+  bool start = true;
+  float gx = bx, gy = by, kp = 0.f, kd = 0.f, wx = 0.f, wy = 0.f, wz = 0.f, eps2 = -1.0f;
+  float caz = 1.f, saz = 0.f, hgrip = 0.f;  // grasp: azimuth of the approach, grip height
   float t_done = (float)T * dt;
-  // Neighbour lists (bit g = geometry g).  A warp rebuilds all its lanes'
-  // lists together as soon as one lane needs it (rebuilding early is always
-  // valid), so the rebuild loop runs once per event instead of once per
-  // lane.  A body left out is at least kSkin away along some axis; a rebuild
-  // once any lane has moved kRebuild keeps it at least 1 cm clear (far above
-  // FP32 rounding), and the later the rebuild, the fewer of them a warp runs.
-  //
-  // Motion budgets: after a contact query that found every listed body
-  // separated, no contact is possible until the mover's path (|dx| + |dy|
-  // (+ |dz|) per step, rounded against it) has used up the smallest gap, so
-  // the queries in between, which would find nothing, are left out.  bclear /
-  // oclear: path left until the next query; bgap / ogap: what the list's own
-  // kRebuild budget is beyond that.  (A position that is not a number leaves
-  // its budgets not numbers and is not queried: its contacts carry no force.)
-  // Measured with the sleeping object and the lanes at rest below: N = 16384
-  // 5.95 -> 5.15 ms, ten iterations of the 64-problem batch 103.7 -> 89.4 ms.
-  constexpr float kSkin = 0.15f, kRebuild = 0.14f;
   unsigned lanes = __activemask();
-  // A* base controller: waypoints of the current moveTo, integral state
+  // A* base controller: goal and waypoints of the current moveTo, integral state
   const bool astar = ASTAR && s.base_ctrl != 0;
   float wpx[kMaxWaypoints], wpy[kMaxWaypoints];
+  float mgx = bx, mgy = by, Ix = 0.f, Iy = 0.f;
   int nwp = 0, wi = 0;
-  float Ix = 0.f, Iy = 0.f;
   bool need_plan = false;
-  uint32_t bmask = 0, omask = 0;
-  float bclear = 0.0f, bgap = 0.0f, oclear = 0.0f, ogap = 0.0f;
+  Reach rb, ro;  // contacts of the base and of the free object
   // asleep: the free object's last step left its position and velocity as
   // they were.  Its step depends on nothing else, so every later one leaves
   // them too, until it is grasped.
   bool asleep = false;
-  bool ik_dirty = true;   // something the inverse kinematics reads changed since it was last solved
-  bool quiet_before = false;
+  bool ik_dirty = true;  // something the inverse kinematics reads changed since it was last solved
+  bool was_quiet = false;
   for (int step = 0; step < T; ++step) {
-    const int ai = a < L ? a : L - 1;
-    const int kind = s.act_kind[ai];
-    if (ai != loaded) {
-      const int o = s.act_off[ai];
-      if (kind == CEM_ACT_MOVE) {
-        mgx = s.act_nom[ai][0] + theta_at(s, row, o);
-        mgy = s.act_nom[ai][1] + theta_at(s, row, o + 1);
-        mkp = theta_at(s, row, o + 2);
-        mkd = 2.0f * sqrtf(mkp);
-        rx = s.act_ref[ai] ? mgx : s.act_nom[ai][0];
-        ry = s.act_ref[ai] ? mgy : s.act_nom[ai][1];
-        if (astar) {  // plan from where the base is now, below, with the whole warp's help
-          need_plan = true;
-          wi = 0;
-          Ix = Iy = 0.f;
-        }
-      } else if (kind == CEM_ACT_GRASP) {
+    if (start) {
+      start = false;
+      ik_dirty = true;
+      kind = s.act_kind[a];
+      const int o = s.act_off[a];
+      eps2 = s.eps * s.eps;
+      if (kind == CEM_ACT_GRASP) {
         sincosf(theta_at(s, row, o), &saz, &caz);
         hgrip = theta_at(s, row, o + 1);
+        if (!(fabsf(hgrip) <= s.grip_tol)) eps2 = -1.0f;  // the gripper never encloses the object
         kp = s.grasp_kp;
         kd = 2.0f * sqrtf(kp);
-      } else if (kind == CEM_ACT_PLACE) {
-        ptx = s.act_nom[ai][0] + theta_at(s, row, o);
-        pty = s.act_nom[ai][1] + theta_at(s, row, o + 1);
-        ptz = s.act_nom[ai][2] + theta_at(s, row, o + 2);
+      } else {
+        if (kind == CEM_ACT_MOVE) {
+          last_move = a;
+        } else {
+          wx = s.act_nom[a][0] + theta_at(s, row, o);
+          wy = s.act_nom[a][1] + theta_at(s, row, o + 1);
+          wz = s.act_nom[a][2] + theta_at(s, row, o + 2);
+        }
+        // the base drives to this moveTo's goal, or holds the last one's
+        gx = s.base_start[0];
+        gy = s.base_start[1];
+        kp = kd = 0.0f;
+        if (last_move >= 0) {
+          const int om = s.act_off[last_move];
+          gx = s.act_nom[last_move][0] + theta_at(s, row, om);
+          gy = s.act_nom[last_move][1] + theta_at(s, row, om + 1);
+          kp = theta_at(s, row, om + 2);
+          kd = 2.0f * sqrtf(kp);
+        }
+        if (kind == CEM_ACT_MOVE) {
+          wx = s.act_ref[a] ? gx : s.act_nom[a][0];
+          wy = s.act_ref[a] ? gy : s.act_nom[a][1];
+          wz = 0.0f;
+          if (astar) {  // plan from where the base is now, below, with the whole warp's help
+            mgx = gx;
+            mgy = gy;
+            need_plan = true;
+            wi = 0;
+            Ix = Iy = 0.f;
+          }
+        }
       }
-      loaded = ai;
-      ik_dirty = true;
     }
     if (astar) {
       // every lane that starts a moveTo this step gets its path in turn: all
@@ -917,144 +1129,128 @@ __device__ __noinline__ void pickplace_rollout(const DevScene& s, const float* _
       }
       need_plan = false;
     }
-    float tx = 0.f, ty = 0.f, tz = 0.f;
     float fix = 0.f, fiy = 0.f;  // integral force per unit mass
-    bool quiet = true;           // nothing of this lane's state changes in this step
-    if (kind == CEM_ACT_MOVE) {
-      gx = mgx;
-      gy = mgy;
-      kp = mkp;
-      kd = mkd;
-      if (astar) {
-        const float Ix0 = Ix, Iy0 = Iy;
-        // past every waypoint already within the switching radius
-        while (wi < nwp - 1 && sqrtf((bx - wpx[wi]) * (bx - wpx[wi]) + (by - wpy[wi]) * (by - wpy[wi])) < s.wp_switch)
-          ++wi;
-        if (wi < nwp - 1) {  // an intermediate waypoint: PD towards it
-          gx = wpx[wi];
-          gy = wpy[wi];
-          Ix = Iy = 0.f;
-        } else {  // the goal: PID, integrating the error near it
-          const float ex_ = mgx - bx, ey_ = mgy - by;
-          if (sqrtf(ex_ * ex_ + ey_ * ey_) < s.pid_irad) {
-            Ix = fminf(fmaxf(Ix + ex_ * dt, -s.pid_imax), s.pid_imax);
-            Iy = fminf(fmaxf(Iy + ey_ * dt, -s.pid_imax), s.pid_imax);
-          } else {
-            Ix = Iy = 0.f;
-          }
-          fix = s.pid_ki * kp * Ix;
-          fiy = s.pid_ki * kp * Iy;
-        }
-        quiet = Ix == Ix0 && Iy == Iy0;
-      }
-    } else if (kind == CEM_ACT_GRASP) {
-      tx = ox;
-      ty = oy;
-      tz = oz + hgrip;
-      gx = ox - s.grasp_reach * caz;
-      gy = oy - s.grasp_reach * saz;
-    } else {
-      tx = ptx;
-      ty = pty;
-      tz = ptz;
-      gx = mgx;
-      gy = mgy;
-      kp = mkp;
-      kd = mkd;
-    }
-    float d2_prev = 0.0f;  // squared distance to the action's target at t_k
-    if (a < L) {
-      if (kind == CEM_ACT_MOVE) d2_prev = (bx - rx) * (bx - rx) + (by - ry) * (by - ry);
-      else d2_prev = (ex - tx) * (ex - tx) + (ey - ty) * (ey - ty) + (ez - tz) * (ez - tz);
-    }
-    if (kind != CEM_ACT_MOVE && ik_dirty) arm_ik<TRACE>(s, bx, by, tx, ty, tz, beta, cbeta, sbeta, q1t, q2t);
-    // base: PD + penalty contacts with the static footprints
-    float fx = mb * (kp * (gx - bx) - kd * bvx);
-    float fy = mb * (kp * (gy - by) - kd * bvy);
+    bool same = true;            // what the step below carries over beside base and arm is unchanged
     if (astar && kind == CEM_ACT_MOVE) {
-      fx += mb * fix;
-      fy += mb * fiy;
-    }
-    if (__any_sync(lanes, bclear <= 0.0f)) {
-      if (__any_sync(lanes, bclear + bgap <= 0.0f)) {
-        bmask = near_list<true, G>(s, n_geoms, bx, by, 0.0f, s.bhx, s.bhy, 0.0f, kSkin, grp);
-        bclear = 0.0f;
-        bgap = kRebuild;
+      const float Ix0 = Ix, Iy0 = Iy;
+      // past every waypoint already within the switching radius
+      while (wi < nwp - 1 && sqrtf((bx - wpx[wi]) * (bx - wpx[wi]) + (by - wpy[wi]) * (by - wpy[wi])) < s.wp_switch)
+        ++wi;
+      gx = mgx;
+      gy = mgy;
+      if (wi < nwp - 1) {  // an intermediate waypoint: PD towards it
+        gx = wpx[wi];
+        gy = wpy[wi];
+        Ix = Iy = 0.f;
+      } else {  // the goal: PID, integrating the error near it
+        const float ex_ = mgx - bx, ey_ = mgy - by;
+        if (sqrtf(ex_ * ex_ + ey_ * ey_) < s.pid_irad) {
+          Ix = fminf(fmaxf(Ix + ex_ * dt, -s.pid_imax), s.pid_imax);
+          Iy = fminf(fmaxf(Iy + ey_ * dt, -s.pid_imax), s.pid_imax);
+        } else {
+          Ix = Iy = 0.f;
+        }
+        fix = s.pid_ki * kp * Ix;
+        fiy = s.pid_ki * kp * Iy;
       }
-      if (bclear <= 0.0f) {
-        float sep = 1e30f;
-        base_contacts<G>(s, bmask, bx, by, bvx, bvy, kc, cc, grp, fx, fy, sep);
-        take_budget(s, sep, fabsf(bx) + fabsf(by), bclear, bgap);
-      }
+      same = Ix == Ix0 && Iy == Iy0;
     }
-    bvx += dt_mb * fx;
-    bvy += dt_mb * fy;
+    if (kind != CEM_ACT_MOVE && ik_dirty) {
+      if (kind == CEM_ACT_GRASP) {
+        wx = ox;
+        wy = oy;
+        wz = oz + hgrip;
+        gx = __fmaf_rn(-s.grasp_reach, caz, ox);
+        gy = __fmaf_rn(-s.grasp_reach, saz, oy);
+      }
+      arm_ik<TRACE>(s, bx, by, wx, wy, wz, beta, cbeta, sbeta, q1t, q2t);
+    }
+    // base: PD + penalty contacts with the static footprints
+    float fx = __fmul_rn(mb, pd_law(kp, gx - bx, kd, bvx));
+    float fy = __fmul_rn(mb, pd_law(kp, gy - by, kd, bvy));
+    if (astar && kind == CEM_ACT_MOVE) {
+      fx = __fmaf_rn(mb, fix, fx);
+      fy = __fmaf_rn(mb, fiy, fy);
+    }
+#ifdef CEM_DEBUG
+    const float fx0 = fx, fy0 = fy;
+#endif
+    if (__any_sync(lanes, rb.due())) {
+      // A warp rebuilds all its lanes' lists together as soon as one lane
+      // needs it (rebuilding early is always valid), so the rebuild loop runs
+      // once per event instead of once per lane.
+      if (__any_sync(lanes, rb.stale()))
+        rb.rebuilt(near_list<true, G>(s, bx, by, 0.0f));
+      // so do the full queries: one lane's takes as long as all lanes'
+      const bool all = __any_sync(lanes, rb.full());
+      if (all || rb.due()) base_contacts<G>(s, rb, all, bx, by, bvx, bvy, kc, cc, fx, fy);
+    }
+#ifdef CEM_DEBUG
+    check_base(s, bx, by, bvx, bvy, kc, cc, fx0, fy0, fx, fy);
+#endif
+    bvx = __fmaf_rn(dt_mb, fx, bvx);
+    bvy = __fmaf_rn(dt_mb, fy, bvy);
     {  // ground friction of the base (yaw is locked)
-      const float v2 = bvx * bvx + bvy * bvy;
-      const float f = v2 > bcap2 ? 1.0f - bcap * rsqrtf(v2) : 0.0f;
-      bvx *= f;
-      bvy *= f;
+      const float v2 = __fmaf_rn(bvx, bvx, __fmul_rn(bvy, bvy));
+      const float f = v2 > bcap2 ? __fmaf_rn(-bcap, rsqrtf(v2), 1.0f) : 0.0f;
+      bvx = __fmul_rn(bvx, f);
+      bvy = __fmul_rn(bvy, f);
     }
     const float bx0 = bx, by0 = by;
-    bx += bvx * dt;
-    by += bvy * dt;
+    bx = __fmaf_rn(bvx, dt, bx);
+    by = __fmaf_rn(bvy, dt, by);
     const float bmoved = __fadd_ru(fabsf(bx - bx0), fabsf(by - by0));
-    bclear = __fadd_rd(bclear, -bmoved);
+    rb.path = __fadd_ru(rb.path, bmoved);
     ik_dirty = bmoved != 0.0f;
     // arm joints
-    const float dd1 = akp * (q1t - q1) - akd * dq1;
-    const float dd2 = akp * (q2t - q2) - akd * dq2;
     const float q10 = q1, q20 = q2, dq10 = dq1, dq20 = dq2;
-    dq1 += dt * dd1;
-    dq2 += dt * dd2;
-    q1 += dt * dq1;
-    q2 += dt * dq2;
-    const bool arm_moved = q1 != q10 || q2 != q20;
-    quiet = quiet && bvx == 0.0f && bvy == 0.0f && !arm_moved && dq1 == dq10 && dq2 == dq20;
-    if (arm_moved) arm_reach(s, q1, q2, fk_r, fk_z);  // the joints as they were: so are reach and height
-    const float nex = bx + fk_r * cbeta, ney = by + fk_r * sbeta, nez = fk_z;
-    // object (a warp-wide rebuild of the object lists, see above)
-    const bool ofree = !attached && !asleep, oquery = ofree && oclear <= 0.0f;
-    if (__any_sync(lanes, oquery)) {
-      const bool rebuild = __any_sync(lanes, oquery && oclear + ogap <= 0.0f);
-      if (rebuild && ofree) {
-        omask = near_list<false, G>(s, n_geoms, ox, oy, oz, h, h, h, kSkin, grp);
-        oclear = 0.0f;
-        ogap = kRebuild;
-      }
-    }
+    dq1 = __fmaf_rn(dt, pd_law(akp, q1t - q1, akd, dq1), dq1);
+    dq2 = __fmaf_rn(dt, pd_law(akp, q2t - q2, akd, dq2), dq2);
+    q1 = __fmaf_rn(dt, dq1, q1);
+    q2 = __fmaf_rn(dt, dq2, q2);
+    float fk_r, fk_z;
+    arm_reach(s, q1, q2, fk_r, fk_z);
+    const float nex = __fmaf_rn(fk_r, cbeta, bx), ney = __fmaf_rn(fk_r, sbeta, by), nez = fk_z;
+    // object
     if (attached) {
       const float ox0 = ox, oy0 = oy, oz0 = oz;
       ox = nex + offx;
       oy = ney + offy;
       oz = nez + offz;
-      const bool held_still = ox == ox0 && oy == oy0 && oz == oz0;
-      quiet = quiet && held_still;
-      ik_dirty = ik_dirty || !held_still;
+      const bool still = ox == ox0 && oy == oy0 && oz == oz0;
+      same = same && still;
+      ik_dirty = ik_dirty || !still;
       if (TRACE) arm_ee_velocity(s, q1, q2, cbeta, sbeta, bvx, bvy, dq1, dq2, ovx, ovy, ovz);
-    } else if (ofree) {
-      const float ox0 = ox, oy0 = oy, oz0 = oz, ovx0 = ovx, ovy0 = ovy, ovz0 = ovz;
-      const bool query = oclear <= 0.0f;
-      float sep = 1e30f;
-      object_contacts<G>(s, op, query ? omask : 0u, ox, oy, oz, ovx, ovy, ovz, kc, cc, grp, sep);
-      if (query) take_budget(s, sep, fabsf(ox) + fabsf(oy) + fabsf(oz), oclear, ogap);
-      ox += ovx * dt;
-      oy += ovy * dt;
-      oz += ovz * dt;
-      oclear = __fadd_rd(oclear, -__fadd_ru(__fadd_ru(fabsf(ox - ox0), fabsf(oy - oy0)), fabsf(oz - oz0)));
-      asleep = ox == ox0 && oy == oy0 && oz == oz0 && ovx == ovx0 && ovy == ovy0 && ovz == ovz0;
-      quiet = quiet && asleep;
-      ik_dirty = ik_dirty || !asleep;  // a grasp aims at the object
     }
-    if (a < L) {
-      float d2_new;
-      if (kind == CEM_ACT_MOVE) d2_new = (bx - rx) * (bx - rx) + (by - ry) * (by - ry);
-      else d2_new = (nex - tx) * (nex - tx) + (ney - ty) * (ney - ty) + (nez - tz) * (nez - tz);
-      bool ok = d2_new <= eps2;
-      if (kind == CEM_ACT_GRASP) ok = ok && fabsf(hgrip) <= s.grip_tol;
-      if (ok) {
-        const float ts = success_time(s, step, sqrtf(d2_prev), sqrtf(d2_new));
-        if (a == L - 1) t_done = ts;
+    const bool ofree = !attached && !asleep;
+    if (__any_sync(lanes, ofree)) {
+      if (__any_sync(lanes, ofree && ro.stale())) {  // as for the base
+        if (ofree) ro.rebuilt(near_list<false, G>(s, ox, oy, oz));
+      }
+      const bool all = __any_sync(lanes, ofree && ro.full());
+      if (ofree) {
+        const float ox0 = ox, oy0 = oy, oz0 = oz, ovx0 = ovx, ovy0 = ovy, ovz0 = ovz;
+        object_contacts<G>(s, op, ro, all || ro.due(), all, ox, oy, oz, ovx, ovy, ovz, kc, cc);
+#ifdef CEM_DEBUG
+        check_object<G>(s, op, ox, oy, oz, ovx0, ovy0, ovz0, ovx, ovy, ovz);
+#endif
+        ox = __fmaf_rn(ovx, dt, ox);
+        oy = __fmaf_rn(ovy, dt, oy);
+        oz = __fmaf_rn(ovz, dt, oz);
+        ro.path = __fadd_ru(ro.path, __fadd_ru(__fadd_ru(fabsf(ox - ox0), fabsf(oy - oy0)), fabsf(oz - oz0)));
+        asleep = ox == ox0 && oy == oy0 && oz == oz0 && ovx == ovx0 && ovy == ovy0 && ovz == ovz0;
+        same = same && asleep;
+        ik_dirty = ik_dirty || !asleep;  // a grasp aims at the object
+      }
+    }
+    const bool move = kind == CEM_ACT_MOVE;
+    {
+      const float dx = (move ? bx : nex) - wx, dy = (move ? by : ney) - wy, dz = move ? 0.0f : nez - wz;
+      const float d2_new = norm2(dx, dy, dz);
+      if (d2_new <= eps2) {
+        // squared distance at t_k
+        const float px = (move ? bx0 : ex) - wx, py = (move ? by0 : ey) - wy, pz = move ? 0.0f : ez - wz;
+        const float ts = success_time(s, step, sqrtf(norm2(px, py, pz)), sqrtf(d2_new));
         if (kind == CEM_ACT_GRASP) {
           attached = true;
           offx = ox - nex;
@@ -1064,12 +1260,17 @@ __device__ __noinline__ void pickplace_rollout(const DevScene& s, const float* _
           if (attached) {  // released with the end effector's velocity (nothing reads it while the object is held)
             if (!TRACE) arm_ee_velocity(s, q1, q2, cbeta, sbeta, bvx, bvy, dq1, dq2, ovx, ovy, ovz);
             asleep = false;
-            oclear = ogap = 0.0f;
+            ro.forget();
           }
           attached = false;
         }
-        ++a;
-        quiet = false;
+        same = false;
+        if (++a < L) {
+          start = true;
+        } else {
+          t_done = ts;
+          eps2 = -1.0f;
+        }
       }
     }
     ex = nex;
@@ -1085,12 +1286,16 @@ __device__ __noinline__ void pickplace_rollout(const DevScene& s, const float* _
     // step mapped the lane's whole state to itself (a step reads nothing else;
     // the step number only enters at an action's end) and every later step
     // would.  The lane leaves with its final state.
-    if (!TRACE && (step & (kQuietEvery - 1)) == kQuietEvery - 1) {
-      const bool done = quiet && quiet_before;
-      lanes = __ballot_sync(lanes, !done);
-      if (done) break;
+    if (!TRACE && (step & (kQuietEvery - 2)) == kQuietEvery - 2) {
+      const bool quiet =
+          same && bvx == 0.0f && bvy == 0.0f && q1 == q10 && q2 == q20 && dq1 == dq10 && dq2 == dq20;
+      if (step & 1) {
+        const bool done = quiet && was_quiet;
+        lanes = __ballot_sync(lanes, !done);
+        if (done) break;
+      }
+      was_quiet = quiet;
     }
-    quiet_before = quiet;
   }
   const bool complete = a == L;
   bool goal = true;
@@ -1382,7 +1587,7 @@ __device__ __forceinline__ void pickplace_batch(const DevScene& s, const float* 
 }
 
 template <int G, bool AS>
-__global__ void __launch_bounds__(256) rollout_persistent_kernel(const DevScene* __restrict__ scenes,
+__global__ void __launch_bounds__(256, 2) rollout_persistent_kernel(const DevScene* __restrict__ scenes,
                                                                  const BatchProblem* __restrict__ probs,
                                                                  const BatchItem* __restrict__ items, int n_items,
                                                                  int* __restrict__ counter,
