@@ -164,7 +164,6 @@ cudaError_t enqueue_screen(cem_batch_ctx* h, cudaStream_t st) {
     cudaError_t e = surrogate_screen_into(h->sur, h->mean_d + (size_t)p * kMS, h->chol_d + (size_t)p * kMC, b.seed,
                                           &h->track_d[p].iter, b.problem, h->n_pool, b.N, h->n_explore, b.D,
                                           h->screen_tab_d + (size_t)p * kTab,
-                                          h->screen_tab_d + (size_t)p * kTab + 2 * CEM_MAX_D,
                                           h->theta_d + b.theta_off, st);
     if (e != cudaSuccess) return e;
   }

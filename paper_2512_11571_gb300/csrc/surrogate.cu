@@ -19,6 +19,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -27,6 +28,7 @@
 
 #include "gelu.cuh"
 #include "internal.h"
+#include "select.cuh"
 
 using namespace cem;
 
@@ -388,24 +390,85 @@ __global__ void to_bf16_kernel(const float* __restrict__ x, size_t n, bf16* __re
   if (i < n) y[i] = __float2bfloat16_rn(x[i]);
 }
 
-// features of N parameter vectors: [clamp(theta) normalised | 0 | scene16]
-template <typename TOut>
-__global__ void features_kernel(const float* __restrict__ theta, int N, int D, const float* __restrict__ lohi,
-                                const float* __restrict__ scene16, TOut* __restrict__ x) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
-  TOut* o = x + (size_t)n * 48;
-  for (int j = 0; j < 48; ++j) {
-    float v = 0.0f;
-    if (j < D) {
-      const float lo = lohi[j], hi = lohi[CEM_MAX_D + j];
-      const float t = fminf(fmaxf(theta[(size_t)n * D + j], lo), hi);
-      v = hi > lo ? (t - 0.5f * (lo + hi)) / (0.5f * (hi - lo)) : 0.0f;
-    } else if (j >= 32) {
-      v = scene16[j - 32];
+// bounds and scene values of one problem's features: lo[18], hi[18], scene[16]
+struct FeatureTable {
+  float lo[CEM_MAX_D], hi[CEM_MAX_D], scene[16];
+};
+static_assert(sizeof(FeatureTable) == sizeof(float) * (2 * CEM_MAX_D + 16), "the layout of the batched screening tables");
+
+__device__ __forceinline__ void store8(float* o, const float* v) {
+  reinterpret_cast<float4*>(o)[0] = make_float4(v[0], v[1], v[2], v[3]);
+  reinterpret_cast<float4*>(o)[1] = make_float4(v[4], v[5], v[6], v[7]);
+}
+__device__ __forceinline__ void store8(bf16* o, const float* v) {
+  __nv_bfloat162 h[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) h[i] = __halves2bfloat162((bf16)v[2 * i], (bf16)v[2 * i + 1]);
+  *reinterpret_cast<uint4*>(o) = *reinterpret_cast<const uint4*>(h);
+}
+
+// features of N parameter vectors: [clamp(theta) normalised | 0 | scene16].
+// One thread per 8 features (six a row), so that a warp writes whole
+// consecutive 16-byte (BF16) or 32-byte pieces; one thread per row wrote 48
+// strided values.  Bound by the bytes written (65,536 rows: 6.3 MB BF16).
+// The table comes by value (tab_d null) or from device memory.  VEC: x is
+// aligned for whole pieces (a caller's FP32 x may not be).
+template <typename TOut, bool VEC>
+__global__ void __launch_bounds__(256) features_kernel(const float* __restrict__ theta, int N, int D,
+                                                       const FeatureTable tab, const FeatureTable* __restrict__ tab_d,
+                                                       TOut* __restrict__ x) {
+  __shared__ FeatureTable sh;  // (lanes of a warp read different entries)
+  {
+    const float* src = tab_d ? reinterpret_cast<const float*>(tab_d) : nullptr;
+    const int i = threadIdx.x;
+    if (i < (int)(sizeof(FeatureTable) / 4)) {
+      const float v = src ? src[i] : i < CEM_MAX_D ? tab.lo[i] : i < 2 * CEM_MAX_D ? tab.hi[i - CEM_MAX_D] : tab.scene[i - 2 * CEM_MAX_D];
+      reinterpret_cast<float*>(&sh)[i] = v;
     }
-    o[j] = (TOut)v;
+    __syncthreads();
   }
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int n = (int)(t / 6), j0 = (int)(t % 6) * 8;
+  if (n >= N) return;
+  float v[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int j = j0 + q;
+    v[q] = 0.0f;
+    if (j < D) {
+      const float lo = sh.lo[j], hi = sh.hi[j];
+      const float c = fminf(fmaxf(theta[(size_t)n * D + j], lo), hi);
+      v[q] = hi > lo ? (c - 0.5f * (lo + hi)) / (0.5f * (hi - lo)) : 0.0f;
+    } else if (j >= 32) {
+      v[q] = sh.scene[j - 32];
+    }
+  }
+  TOut* o = x + (size_t)n * 48 + j0;
+  if (VEC) {
+    store8(o, v);
+  } else {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) o[q] = (TOut)v[q];
+  }
+}
+
+template <typename TOut>
+cudaError_t features(const float* theta, int N, int D, const FeatureTable& tab, const FeatureTable* tab_d, TOut* x,
+                     cudaStream_t st) {
+  const unsigned grid = (unsigned)(((long long)N * 6 + 255) / 256);
+  if (((uintptr_t)x & 15u) == 0) features_kernel<TOut, true><<<grid, 256, 0, st>>>(theta, N, D, tab, tab_d, x);
+  else features_kernel<TOut, false><<<grid, 256, 0, st>>>(theta, N, D, tab, tab_d, x);
+  return cudaGetLastError();
+}
+
+FeatureTable feature_table(int D, const float* lo, const float* hi, const float* scene16) {
+  FeatureTable t;
+  for (int d = 0; d < CEM_MAX_D; ++d) {
+    t.lo[d] = d < D ? lo[d] : 0.0f;
+    t.hi[d] = d < D ? hi[d] : 0.0f;
+  }
+  for (int i = 0; i < 16; ++i) t.scene[i] = scene16[i];
+  return t;
 }
 
 // minibatch of B rows drawn with replacement (Philox on (step, i)); gathers x and t
@@ -438,99 +501,141 @@ __global__ void gather_batch_kernel(const bf16* __restrict__ X, const float* __r
 }
 
 // ---------------------------------------------------------------- top-k
-__device__ __forceinline__ uint32_t order_bits(float x) {
-  const uint32_t u = __float_as_uint(x);
-  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-__device__ __forceinline__ uint64_t score_key(const float* s, int i) {
-  float v = s[i];
-  if (!isfinite(v)) v = __int_as_float(0x7f800000);
-  v = v + 0.0f;
-  return ((uint64_t)order_bits(v) << 20) | (uint64_t)i;
-}
+// Indices of the `keep` lowest scores (ties by index), in ascending index
+// order; scores that are not finite come last, and the first n_explore
+// entries count as the lowest finite score whatever theirs is (unscreened
+// draws from the current distribution).  One cluster: CTA c owns the c-th
+// contiguous share of the array, thread t every 1024th element of it, so
+// that (round, thread) order is index order: after the radix select the
+// kept ones are numbered by ballots, a scan over (round, warp) counts and the
+// other CTAs' totals.  Bound by the latency of its few rounds and cluster
+// barriers: 65,536 scores took 150 us in one CTA, see launch_topk.
+constexpr int kTopkRegs = 8;  // keys per thread kept in registers
+constexpr int kTopkRounds = CEM_MAX_N / (8 * kSelThreads);
 
-// indices of the `keep` lowest scores (ties by index), written in ascending
-// index order; one CTA of 1024 threads (radix select, then an ordered scan)
-__global__ void __launch_bounds__(1024) topk_kernel(const float* __restrict__ score, int N, int keep,
-                                                    int32_t* __restrict__ idx) {
-  __shared__ uint32_t hist[256];
-  __shared__ uint64_t s_prefix, s_mask;
-  __shared__ int s_rank;
-  __shared__ int warp_tot[32];
-  const int tid = threadIdx.x;
-  if (tid == 0) {
-    s_prefix = 0;
-    s_mask = 0;
-    s_rank = keep;
-  }
-  __syncthreads();
-  uint64_t kth = ~0ull;
+__global__ void __launch_bounds__(kSelThreads) topk_kernel(const float* __restrict__ score, int N, int n_explore,
+                                                           int keep, int32_t* __restrict__ idx) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  __shared__ SelectShared sh;
+  extern __shared__ __align__(8) uint32_t rounds_sm[];  // per (round, warp): kept below the cut, ties
+  __shared__ __align__(8) uint32_t total[2];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int nc = (int)cl.num_blocks(), c = (int)cl.block_rank();
+  const int rounds = (N + nc * kSelThreads - 1) / (nc * kSelThreads);
+  const int first = c * rounds * kSelThreads;
+  auto key_at = [&](int j) -> uint32_t {
+    const int i = first + j * kSelThreads + tid;
+    if (i >= N) return 0xffffffffu;
+    float v = score[i];
+    if (!isfinite(v)) v = __int_as_float(0x7f800000);
+    if (i < n_explore) v = -3.402823466e38f;
+    return float_order(v);
+  };
+  uint32_t rk[kTopkRegs];
+#pragma unroll
+  for (int j = 0; j < kTopkRegs; ++j) rk[j] = j < rounds ? key_at(j) : 0xffffffffu;
+  auto each = [&](auto f) {
+#pragma unroll
+    for (int j = 0; j < kTopkRegs; ++j)
+      if (j < rounds) f(first + j * kSelThreads + tid < N, rk[j]);
+    for (int j = kTopkRegs; j < rounds; ++j) f(first + j * kSelThreads + tid < N, key_at(j));
+  };
+  Cut cut{0xffffffffu, N};
   if (keep < N) {
-    int shift = 52;
-    while (shift > 0) {
-      const int width = shift >= 8 ? 8 : shift;
-      shift -= width;
-      for (int d = tid; d < 256; d += 1024) hist[d] = 0;
-      __syncthreads();
-      const uint64_t prefix = s_prefix, mask = s_mask;
-      for (int i = tid; i < N; i += 1024) {
-        const uint64_t key = score_key(score, i);
-        if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & ((1u << width) - 1)], 1u);
-      }
-      __syncthreads();
-      if (tid == 0) {
-        uint32_t cum = 0;
-        int d = 0;
-        for (; d < (1 << width); ++d) {
-          if (cum + hist[d] >= (uint32_t)s_rank) break;
-          cum += hist[d];
-        }
-        s_rank -= (int)cum;
-        s_prefix |= (uint64_t)d << shift;
-        s_mask |= (uint64_t)((1u << width) - 1) << shift;
-      }
-      __syncthreads();
+    select_clear(sh);
+    __syncthreads();
+    cut = cluster_select(cl, sh, each, (uint32_t)keep);
+  }
+  // kept elements per (round, warp): below the cut in the low, ties in the high half of a pair of words
+  uint32_t* below = rounds_sm;
+  uint32_t* ties = rounds_sm + rounds * 32;
+  int j = 0;
+  each([&](bool valid, uint32_t key) {
+    const unsigned bl = __ballot_sync(0xffffffffu, valid && key < cut.key);
+    const unsigned bt = __ballot_sync(0xffffffffu, valid && key == cut.key);
+    if (lane == 0) {
+      below[j * 32 + w] = (uint32_t)__popc(bl);
+      ties[j * 32 + w] = (uint32_t)__popc(bt);
     }
-    kth = s_prefix;
-  }
-  // ordered compaction: thread tid owns the contiguous range [tid*per, (tid+1)*per)
-  const int per = (N + 1023) / 1024;
-  const int b = tid * per, e = min(N, b + per);
-  int cnt = 0;
-  for (int i = b; i < e; ++i) cnt += score_key(score, i) <= kth;
-  // exclusive scan of cnt over the block
-  int x = cnt;
-  const int lane = tid & 31, w = tid >> 5;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) warp_tot[w] = x;
+    ++j;
+  });
   __syncthreads();
-  if (w == 0) {
-    int t = warp_tot[lane];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, t, o);
-      if (lane >= o) t += y;
-    }
-    warp_tot[lane] = t;
+  // exclusive scans over the (round, warp) counts, each thread a run of them
+  const int cells = rounds * 32, per = (cells + kSelThreads - 1) / kSelThreads;
+  uint32_t sb = 0, st = 0;
+  for (int q = tid * per; q < min(cells, (tid + 1) * per); ++q) {
+    sb += below[q];
+    st += ties[q];
   }
+  const uint32_t ib = block_scan(sb, sh.warp_sum);
   __syncthreads();
-  int pos = x - cnt + (w > 0 ? warp_tot[w - 1] : 0);
-  for (int i = b; i < e; ++i)
-    if (score_key(score, i) <= kth) {
-      if (pos < keep) idx[pos] = i;
-      ++pos;
+  const uint32_t it = block_scan(st, sh.warp_sum);
+  if (tid == kSelThreads - 1) {
+    total[0] = ib;
+    total[1] = it;
+  }
+  uint32_t xb = ib - sb, xt = it - st;
+  for (int q = tid * per; q < min(cells, (tid + 1) * per); ++q) {
+    const uint32_t vb = below[q], vt = ties[q];
+    below[q] = xb;
+    ties[q] = xt;
+    xb += vb;
+    xt += vt;
+  }
+  if (nc > 1) cl.sync();
+  else __syncthreads();
+  uint32_t ob = 0, ot = 0;  // kept by the CTAs before this one
+#pragma unroll
+  for (int r = 0; r < kSelCtas - 1; ++r)
+    if (r < c) {
+      const uint2 t = *reinterpret_cast<const uint2*>(cl.map_shared_rank(&total[0], r));
+      ob += t.x;
+      ot += t.y;
     }
+  const uint32_t take = (uint32_t)cut.take;
+  j = 0;
+  each([&](bool valid, uint32_t key) {
+    const bool lo = valid && key < cut.key, eq = valid && key == cut.key;
+    const unsigned bl = __ballot_sync(0xffffffffu, lo), bt = __ballot_sync(0xffffffffu, eq);
+    const unsigned lt = (1u << lane) - 1u;
+    const uint32_t nb = ob + below[j * 32 + w] + (uint32_t)__popc(bl & lt);
+    const uint32_t nt = ot + ties[j * 32 + w] + (uint32_t)__popc(bt & lt);
+    if (lo || (eq && nt < take)) {
+      const uint32_t pos = nb + min(nt, take);
+      if (pos < (uint32_t)keep) idx[pos] = first + j * kSelThreads + tid;
+    }
+    ++j;
+  });
+  if (nc > 1) cl.sync();  // the totals stay until every CTA has read them
 }
 
-// the first n_explore pool entries are kept whatever their score (unscreened
-// draws from the current distribution): give them the lowest finite score
-__global__ void force_keep_kernel(float* __restrict__ score, int n_explore) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n_explore) score[i] = -3.402823466e38f;
+cudaError_t launch_topk(const float* score, int N, int n_explore, int keep, int32_t* idx, cudaStream_t st) {
+  const int nc = select_ctas(N), rounds = (N + nc * kSelThreads - 1) / (nc * kSelThreads);
+  constexpr int kMaxDevices = 64;
+  static std::atomic<bool> configured[kMaxDevices];  // host threads may race here; the set-up is idempotent
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  if (!configured[dev].load(std::memory_order_acquire)) {
+    e = cudaFuncSetAttribute(topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(uint32_t) * 2 * 32 * kTopkRounds);
+    if (e != cudaSuccess) return e;
+    configured[dev].store(true, std::memory_order_release);
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)nc);
+  cfg.blockDim = dim3(kSelThreads);
+  cfg.dynamicSmemBytes = sizeof(uint32_t) * 2 * 32 * (size_t)rounds;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)nc;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, topk_kernel, score, N, n_explore, keep, idx);
 }
 
 // training target of a simulated sample: log(1 + max(J, 0) + 10 * class),
@@ -691,8 +796,6 @@ struct cem_surrogate_ctx {
   bf16* pool_x = nullptr;
   float* pool_score = nullptr;
   int32_t* keep_idx = nullptr;
-  float* lohi = nullptr;
-  float* scene16 = nullptr;
   // fused tcgen05 forward: packed weights (rebuilt when the BF16 weights
   // change), status word of its bounded waits, path selection
   void* tc_pack = nullptr;
@@ -1098,8 +1201,6 @@ int cem_surrogate_create(int in_dim, int width, int depth, uint64_t seed, cem_su
   A((void**)&s->m1, sizeof(float) * o);
   A((void**)&s->m2, sizeof(float) * o);
   A((void**)&s->norm, sizeof(float) * 2);
-  A((void**)&s->lohi, sizeof(float) * 2 * CEM_MAX_D);
-  A((void**)&s->scene16, sizeof(float) * 16);
   if (mlp_tc_supported(in_dim, width, depth)) A(&s->tc_pack, mlp_tc_pack_bytes());
   A((void**)&s->tc_status, sizeof(int));
   A((void**)&s->step_d, sizeof(int));
@@ -1127,7 +1228,7 @@ int cem_surrogate_destroy(cem_surrogate_handle s) {
   if (!s) return CEM_OK;
   cudaDeviceSynchronize();
   sur_free_work(s);
-  void* ptrs[] = {s->p, s->pb, s->g, s->m1, s->m2, s->norm, s->lohi, s->scene16,
+  void* ptrs[] = {s->p, s->pb, s->g, s->m1, s->m2, s->norm,
                   s->pool_theta, s->pool_x, s->pool_score, s->keep_idx, s->tc_pack, s->tc_status,
                   s->step_d, s->adam_t_d};
   for (void* p : ptrs) cudaFree(p);
@@ -1360,16 +1461,8 @@ int cem_surrogate_features(cem_surrogate_handle s, const float* theta_d, int N, 
   if (N == 0) return CEM_OK;
   if (!is_dev(theta_d) || !is_dev(x_d)) return fail(CEM_ERR_INVALID_ARG, "theta and x must be device pointers");
   cudaStream_t st = (cudaStream_t)stream;
-  float tab[2 * CEM_MAX_D];
-  for (int d = 0; d < CEM_MAX_D; ++d) {
-    tab[d] = d < D ? lo_h[d] : 0.0f;
-    tab[CEM_MAX_D + d] = d < D ? hi_h[d] : 0.0f;
-  }
-  SUR_CUDA(cudaMemcpyAsync(s->lohi, tab, sizeof(tab), cudaMemcpyHostToDevice, st));
-  SUR_CUDA(cudaMemcpyAsync(s->scene16, scene16_h, sizeof(float) * 16, cudaMemcpyHostToDevice, st));
-  features_kernel<float><<<(N + 127) / 128, 128, 0, st>>>(theta_d, N, D, s->lohi, s->scene16, x_d);
-  SUR_CUDA(cudaGetLastError());
-  SUR_CUDA(cudaStreamSynchronize(st));  // the host tables are consumed
+  SUR_CUDA(features<float>(theta_d, N, D, feature_table(D, lo_h, hi_h, scene16_h), nullptr, x_d, st));
+  SUR_CUDA(cudaStreamSynchronize(st));  // as ever: the features are complete when the call returns
   return CEM_OK;
 }
 
@@ -1403,42 +1496,22 @@ int ensure_pool(cem_surrogate_ctx* s, int P, int N, int D) {
 }
 
 // pool theta (already sampled, P x D) -> scores -> indices of the N best ->
-// theta_keep (N x D), all on `st`; features from the bounds lohi[2 x 18]
-// and the scene values scene16[16] (device)
-cudaError_t screen_pool_tab(cem_surrogate_ctx* s, int P, int N, int n_explore, int D, const float* lohi,
-                            const float* scene16, float* theta_keep, cudaStream_t st) {
-  features_kernel<bf16><<<(P + 127) / 128, 128, 0, st>>>(s->pool_theta, P, D, lohi, scene16, s->xin);
-  cudaError_t e = cudaGetLastError();
+// theta_keep (N x D), all on `st`; the features' table by value, or tab_d on
+// the device
+cudaError_t screen_pool(cem_surrogate_ctx* s, int P, int N, int n_explore, int D, const FeatureTable& tab,
+                        const FeatureTable* tab_d, float* theta_keep, cudaStream_t st) {
+  cudaError_t e = features<bf16>(s->pool_theta, P, D, tab, tab_d, s->xin, st);
   if (e != cudaSuccess) return e;
   e = infer_rows(s, P, s->pool_score, st);
   if (e != cudaSuccess) return e;
-  if (n_explore > 0) {
-    force_keep_kernel<<<(n_explore + 255) / 256, 256, 0, st>>>(s->pool_score, n_explore);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  topk_kernel<<<1, 1024, 0, st>>>(s->pool_score, P, N, s->keep_idx);
-  e = cudaGetLastError();
+  e = launch_topk(s->pool_score, P, n_explore, N, s->keep_idx, st);
   if (e != cudaSuccess) return e;
   gather_rows_kernel<<<(N * D + 255) / 256, 256, 0, st>>>(s->pool_theta, P, s->keep_idx, N, D, theta_keep);
   return cudaGetLastError();
 }
 
-cudaError_t screen_pool(cem_surrogate_ctx* s, int P, int N, int n_explore, int D, float* theta_keep,
-                        cudaStream_t st) {
-  return screen_pool_tab(s, P, N, n_explore, D, s->lohi, s->scene16, theta_keep, st);
-}
-
-int set_tables(cem_surrogate_ctx* s, const cem_skeleton_desc& k, const float* scene16_h, cudaStream_t st) {
-  float tab[2 * CEM_MAX_D];
-  for (int d = 0; d < CEM_MAX_D; ++d) {
-    tab[d] = d < k.D ? k.lo[d] : 0.0f;
-    tab[CEM_MAX_D + d] = d < k.D ? k.hi[d] : 0.0f;
-  }
-  SUR_CUDA(cudaMemcpyAsync(s->lohi, tab, sizeof(tab), cudaMemcpyHostToDevice, st));
-  SUR_CUDA(cudaMemcpyAsync(s->scene16, scene16_h, sizeof(float) * 16, cudaMemcpyHostToDevice, st));
-  SUR_CUDA(cudaStreamSynchronize(st));
-  return CEM_OK;
+FeatureTable skeleton_table(const cem_skeleton_desc& k, const float* scene16_h) {
+  return feature_table(k.D, k.lo, k.hi, scene16_h);
 }
 
 }  // namespace
@@ -1457,11 +1530,12 @@ int surrogate_reserve_pool(cem_surrogate_handle s, int n_pool, int n_keep, int D
 
 cudaError_t surrogate_screen_into(cem_surrogate_handle s, const float* mean, const float* chol, uint64_t seed,
                                   const uint32_t* iter_ptr, uint32_t problem, int n_pool, int n_keep, int n_explore,
-                                  int D, const float* lohi, const float* scene16, float* theta_keep,
-                                  cudaStream_t st) {
+                                  int D, const float* tab, float* theta_keep, cudaStream_t st) {
   cudaError_t e = launch_sample(mean, chol, seed, iter_ptr, 0, problem, n_pool, D, s->pool_theta, st);
   if (e != cudaSuccess) return e;
-  return screen_pool_tab(s, n_pool, n_keep, n_explore, D, lohi, scene16, theta_keep, st);
+  // (lo[18], hi[18], scene[16] are contiguous in the batch's table)
+  return screen_pool(s, n_pool, n_keep, n_explore, D, FeatureTable{}, reinterpret_cast<const FeatureTable*>(tab), theta_keep,
+                     st);
 }
 
 int surrogate_status_word(cem_surrogate_handle s) {
@@ -1488,10 +1562,8 @@ int cem_surrogate_screen(cem_handle h, cem_surrogate_handle s, const float* mean
   cudaStream_t st = (cudaStream_t)stream;
   int rc = ensure_pool(s, n_pool, n_keep, k.D);
   if (rc != CEM_OK) return rc;
-  rc = set_tables(s, k, scene16_h, st);
-  if (rc != CEM_OK) return rc;
   SUR_CUDA(launch_sample(mean_d, chol_d, seed, nullptr, iter, problem, n_pool, k.D, s->pool_theta, st));
-  SUR_CUDA(screen_pool(s, n_pool, n_keep, 0, k.D, theta_keep_d, st));
+  SUR_CUDA(screen_pool(s, n_pool, n_keep, 0, k.D, skeleton_table(k, scene16_h), nullptr, theta_keep_d, st));
   if (keep_idx_d)
     SUR_CUDA(cudaMemcpyAsync(keep_idx_d, s->keep_idx, sizeof(int32_t) * n_keep, cudaMemcpyDeviceToDevice, st));
   return CEM_OK;
@@ -1543,8 +1615,7 @@ int solve_screened(cem_handle h, cem_surrogate_handle s, const float* scene16_h,
   rc = handle_solve_buffers(h, N, p->iters, &b);
   if (rc != CEM_OK) return rc;
   cudaStream_t st = b.stream;
-  rc = set_tables(s, k, scene16_h, st);
-  if (rc != CEM_OK) return rc;
+  const FeatureTable tab = skeleton_table(k, scene16_h);
   rc = handle_init_distribution(h, p, &b);
   if (rc != CEM_OK) return rc;
   RefitArgs a;
@@ -1572,7 +1643,7 @@ int solve_screened(cem_handle h, cem_surrogate_handle s, const float* scene16_h,
   SUR_CUDA(cudaEventRecord(b.ev0, st));
   for (int j = 0; j < p->iters; ++j) {
     SUR_CUDA(launch_sample(b.mean, b.chol, p->seed, &b.track->iter, 0, p->problem, n_pool, D, s->pool_theta, st));
-    SUR_CUDA(screen_pool(s, n_pool, N, n_explore, D, b.theta, st));
+    SUR_CUDA(screen_pool(s, n_pool, N, n_explore, D, tab, nullptr, b.theta, st));
     DrArgs dr;
     if (b.dr) {
       dr = *b.dr;
@@ -1582,7 +1653,7 @@ int solve_screened(cem_handle h, cem_surrogate_handle s, const float* scene16_h,
     SUR_CUDA(launch_rollout(b.scene, b.kind, b.theta, N, b.J, b.cls, b.block, b.tpr, b.dr ? &dr : nullptr, st, b.astar));
     if (ft) {  // this iteration's simulated samples (features, score targets) into the ring
       const int pos = (int)(((long long)j * N) % ft->capacity);
-      features_kernel<float><<<(N + 127) / 128, 128, 0, st>>>(b.theta, N, D, s->lohi, s->scene16, rb.x + (size_t)pos * 48);
+      SUR_CUDA(features<float>(b.theta, N, D, tab, nullptr, rb.x + (size_t)pos * 48, st));
       score_target_kernel<<<(N + 255) / 256, 256, 0, st>>>(b.J, b.cls, N, rb.t + pos);
       SUR_CUDA(cudaGetLastError());
     }
