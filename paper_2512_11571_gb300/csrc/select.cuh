@@ -29,17 +29,18 @@ constexpr int kSelCtas = 8;  // the largest cluster
 // most four, then enough to keep eight a thread in registers, up to eight
 inline int select_ctas(int n) { return n <= 4 * kSelThreads ? 1 : n <= 16 * kSelThreads ? 4 : kSelCtas; }
 
-// the keys below `key` and `take` of those equal to it are the wanted ones
+// the keys below `key` and `take` of the `equal` ones that equal it are the
+// wanted ones
 struct Cut {
   uint32_t key;
-  int take;
+  int take, equal;
 };
 
 struct SelectShared {
   uint32_t hist[kSelPasses][kSelBins];
   uint32_t warp_sum[32];
   uint2 range;  // smallest and largest key of this CTA
-  uint32_t bin, before;
+  uint32_t bin, before, in_bin;
 };
 
 // order-preserving bits of a float (a negative zero counts as zero)
@@ -82,7 +83,7 @@ template <class Each>
 __device__ __forceinline__ Cut cluster_select(cooperative_groups::cluster_group& cl, SelectShared& sh, Each each,
                                               uint32_t need) {
   const int tid = threadIdx.x, lane = tid & 31, nc = (int)cl.num_blocks();
-  uint32_t lo = 0xffffffffu, hi = 0u;
+  uint32_t lo = 0xffffffffu, hi = 0u, equal = 0u;
   each([&](bool valid, uint32_t key) {
     if (valid) {
       lo = min(lo, key);
@@ -139,15 +140,17 @@ __device__ __forceinline__ Cut cluster_select(cooperative_groups::cluster_group&
       const bool second = need > excl + a;
       sh.bin = (uint32_t)(2 * tid) + (second ? 1u : 0u);
       sh.before = excl + (second ? a : 0u);
+      sh.in_bin = second ? b : a;
     }
     __syncthreads();
     lo += sh.bin << shift;
     hi = min(hi, lo + ((1u << shift) - 1u));
     need -= sh.before;
+    equal = sh.in_bin;
     __syncthreads();
     if (shift == 0) break;  // (the same in every thread of the cluster)
   }
-  return Cut{lo, (int)need};
+  return Cut{lo, (int)need, (int)equal};
 }
 
 }  // namespace cem

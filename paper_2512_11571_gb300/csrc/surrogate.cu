@@ -541,7 +541,7 @@ __global__ void __launch_bounds__(kSelThreads) topk_kernel(const float* __restri
       if (j < rounds) f(first + j * kSelThreads + tid < N, rk[j]);
     for (int j = kTopkRegs; j < rounds; ++j) f(first + j * kSelThreads + tid < N, key_at(j));
   };
-  Cut cut{0xffffffffu, N};
+  Cut cut{0xffffffffu, N, 0};
   if (keep < N) {
     select_clear(sh);
     __syncthreads();
