@@ -24,7 +24,7 @@
 // What bounds it: latency, and the FP64 units for the statistics (about two
 // multiply-adds per cycle and SM: 105 sums of 512 at D = 14 are 27,000 cycles
 // in one CTA).  N = 16384, K = 512, D = 14 in one CTA, seven 8-bit passes with
-// match.any, one FP64 sum per four threads: 75 us; here: see launch_refit.
+// match.any, one FP64 sum per four threads: 90 us (ncu, cold); here 47 us.
 #include "internal.h"
 #include "select.cuh"
 
@@ -59,12 +59,16 @@ __device__ __forceinline__ int classify(const float* __restrict__ J, const uint8
 
 __device__ __forceinline__ uint64_t elite_key(uint32_t key, int i) { return ((uint64_t)key << 20) | (uint64_t)i; }
 
-__device__ bool cholesky_warp(double* A, int D, int lane) {
-  // right-looking, in place, lower triangle; lane i owns row i
+// right-looking Cholesky factor in place, lower triangle, by one warp: the
+// trailing update of a column is spread over the lanes element by element
+// (a row per lane left the chain of one row's updates, 1800 cycles a column
+// at D = 14)
+// (tri[t] = 32 p + q for t = p (p + 1) / 2 + q, q <= p)
+constexpr int kTri = (CEM_MAX_D - 1) * CEM_MAX_D / 2;
+__device__ bool cholesky_warp(double* A, int D, int lane, const uint16_t* tri) {
   for (int j = 0; j < D; ++j) {
-    double d = A[j * D + j];
-    const bool ok = d > 0.0;
-    if (!__all_sync(0xffffffffu, ok)) return false;
+    const double d = A[j * D + j];
+    if (!__all_sync(0xffffffffu, d > 0.0)) return false;
     // one reciprocal square root instead of a square root and a division
     // per row (FP64 is slow on this part; the result is cast to FP32)
     const double r = rsqrt(d);
@@ -73,8 +77,12 @@ __device__ bool cholesky_warp(double* A, int D, int lane) {
     if (lane == j) A[j * D + j] = ljj;
     if (lane > j && lane < D) A[lane * D + j] *= r;
     __syncwarp();
-    if (lane > j && lane < D)
-      for (int k = j + 1; k <= lane; ++k) A[lane * D + k] -= A[lane * D + j] * A[k * D + j];
+    // elements (j + 1 + p, j + 1 + q), q <= p, of the trailing triangle
+    const int m = D - 1 - j;
+    for (int t = lane; t < m * (m + 1) / 2; t += 32) {
+      const int i = j + 1 + (tri[t] >> 5), k = j + 1 + (tri[t] & 31);
+      A[i * D + k] -= A[i * D + j] * A[k * D + j];
+    }
     __syncwarp();
   }
   return true;
@@ -141,6 +149,7 @@ __device__ __forceinline__ void refit_body(const RefitArgs& a) {
   __shared__ double s_mean[CEM_MAX_D];
   __shared__ double s_cov[CEM_MAX_D * CEM_MAX_D];
   __shared__ double s_L[CEM_MAX_D * CEM_MAX_D];
+  __shared__ uint16_t s_tri[kTri];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, N = a.N, D = a.D;
   const int nc = (int)cl.num_blocks(), c = (int)cl.block_rank();
   auto sync_all = [&]() {
@@ -151,6 +160,11 @@ __device__ __forceinline__ void refit_body(const RefitArgs& a) {
   if (tid < 4) cnt[tid] = 0;
   if (tid == 0) s_n = 0;
   select_clear(sh);
+  if (tid < kTri) {
+    int p = 0;
+    while ((p + 1) * (p + 2) / 2 <= tid) ++p;
+    s_tri[tid] = (uint16_t)(32 * p + tid - p * (p + 1) / 2);
+  }
   __syncthreads();
   // this CTA's samples: c, c + nc, ... in runs of 1024; their keys and classes
   // (4: no sample), the first KR rounds in registers
@@ -238,7 +252,8 @@ __device__ __forceinline__ void refit_body(const RefitArgs& a) {
       }
       __syncthreads();
     } else {
-      Cut cut{0xffffffffu, 0, 0}, tie{0xffffffffu, 0, 0};
+      Cut cut{0xffffffffu, 0, 0};
+      uint32_t tie_end = 0xffffffffu;  // samples of the cut's cost up to this index (exclusive)
       if (keff < in_class) {
         cut = cluster_select(cl, sh, [&](auto f) { each([&](int, int k, uint32_t key) { f(k == cstar, key); }); },
                              (uint32_t)keff);
@@ -246,33 +261,60 @@ __device__ __forceinline__ void refit_body(const RefitArgs& a) {
           sync_all();
           select_clear(sh);
           __syncthreads();
-          tie = cluster_select(cl, sh, [&](auto f) {
+          const Cut t = cluster_select(cl, sh, [&](auto f) {
             each([&](int i, int k, uint32_t key) { f(k == cstar && key == cut.key, (uint32_t)i); });
           }, (uint32_t)cut.take);
+          tie_end = t.key + (t.take > 0 ? 1u : 0u);
         }
       }
-      // gather the elites in the first CTA (unordered), then sort them there
-      if (c == 0)
+      // gather the elites (unordered), then sort them: in a cluster every CTA
+      // gets all of them and ranks its share by counting, a single CTA (or more
+      // than 1024 elites) sorts them in the first one
+      const bool count = nc > 1 && keff <= RT;
+      uint64_t* bag = count ? reinterpret_cast<uint64_t*>(&sh.hist[0][0]) : keys;
+      if (!count && c == 0)
         for (int i = tid; i < P; i += RT) keys[i] = ~0ull;
-      sync_all();
+      sync_all();  // (nobody reads this CTA's histograms any more)
       int* n0 = at0(&s_n);
-      uint64_t* keys0 = at0(keys);
+      uint64_t* bag0 = at0(bag);
       each([&](int i, int k, uint32_t key) {
-        const bool in = k == cstar && (key < cut.key || (key == cut.key && (uint32_t)i <= tie.key));
+        const bool in = k == cstar && (key < cut.key || (key == cut.key && (uint32_t)i < tie_end));
         const unsigned m = __ballot_sync(0xffffffffu, in);
         if (m == 0u) return;
         int pos = 0;
         if (lane == __ffs(m) - 1) pos = atomicAdd(n0, __popc(m));
         pos = __shfl_sync(0xffffffffu, pos, __ffs(m) - 1) + __popc(m & ((1u << lane) - 1u));
-        if (in && pos < P) keys0[pos] = elite_key(key, i);
+        if (in && pos < P) {
+          if (count)
+            for (int r = 0; r < nc; ++r) cl.map_shared_rank(bag, r)[pos] = elite_key(key, i);
+          else
+            bag0[pos] = elite_key(key, i);
+        }
       });
       sync_all();
-      if (c == 0) sort_keys(keys, P);
-      if (nc > 1) {  // every CTA takes the sorted keys
+      if (count) {
+        const int per = (keff + nc - 1) / nc;  // elites e = c per .. of this CTA, tpk threads each
+        int tpk = 32;
+        while (tpk * per > RT) tpk >>= 1;
+        const int e = c * per + tid / tpk;
+        const bool mine = tid / tpk < per && e < keff;
+        const uint64_t key = mine ? bag[e] : 0ull;
+        int rank = 0;
+        if (mine)
+#pragma unroll 8
+          for (int q = tid & (tpk - 1); q < keff; q += tpk) rank += bag[q] < key;
+        for (int o = tpk >> 1; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+        if (mine)
+          for (int r = tid & (tpk - 1); r < nc; r += tpk) cl.map_shared_rank(keys, r)[rank] = key;
         cl.sync();
-        if (c > 0)
-          for (int i = tid; i < keff; i += RT) keys[i] = keys0[i];
-        __syncthreads();
+      } else {
+        if (c == 0) sort_keys(keys, P);
+        if (nc > 1) {  // every CTA takes the sorted keys
+          cl.sync();
+          if (c > 0)
+            for (int i = tid; i < keff; i += RT) keys[i] = bag0[i];
+          __syncthreads();
+        }
       }
     }
     if (c == 0 && a.elite_idx)
@@ -299,10 +341,19 @@ __device__ __forceinline__ void refit_body(const RefitArgs& a) {
       const double invk = 1.0 / (double)keff;
       double* X = reinterpret_cast<double*>(dyn + sizeof(uint64_t) * (size_t)P);
       if (staged) {
-        for (int q = tid; q < keff * D; q += RT) {
-          const int e = q / D, d = q - e * D;
-          X[d * keff + e] = (double)eth(e, d);
+        // two threads per elite, the loads of half a row in flight together
+        constexpr int HALF = (CEM_MAX_D + 1) / 2;
+        const int e = tid >> 1, d0 = (tid & 1) * HALF;
+        if (e < keff) {
+          const float* row = a.theta + (size_t)CEM_DIDX((int)(keys[e] & 0xFFFFF), a.N, 8) * D;
+          float v[HALF];
+#pragma unroll
+          for (int q = 0; q < HALF; ++q) v[q] = d0 + q < D ? row[d0 + q] : 0.0f;
+#pragma unroll
+          for (int q = 0; q < HALF; ++q)
+            if (d0 + q < D) X[(d0 + q) * keff + e] = (double)v[q];
         }
+        static_assert(2 * KSTAGE <= RT, "two threads per staged elite");
         __syncthreads();
       }
       // a warp per output, lane l adding e = l, l + 32, ..., then a butterfly;
@@ -362,7 +413,7 @@ __device__ __forceinline__ void refit_body(const RefitArgs& a) {
     if (tid < 32) {
       for (int i = tid; i < D * D; i += 32) s_L[i] = (i % D) <= (i / D) ? s_cov[i] : 0.0;
       __syncwarp();
-      bool ok = cholesky_warp(s_L, D, tid);
+      bool ok = cholesky_warp(s_L, D, tid, s_tri);
       if (!ok) {  // fall back to the diagonal
         for (int i = tid; i < D * D; i += 32) {
           const bool dg = i / D == i % D;
@@ -370,7 +421,7 @@ __device__ __forceinline__ void refit_body(const RefitArgs& a) {
           s_L[i] = dg ? s_cov[i] : 0.0;
         }
         __syncwarp();
-        ok = cholesky_warp(s_L, D, tid);
+        ok = cholesky_warp(s_L, D, tid, s_tri);
       }
       if (tid == 0) s_fail = ok ? 0 : 1;
     }

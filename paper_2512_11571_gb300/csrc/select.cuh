@@ -29,8 +29,8 @@ constexpr int kSelCtas = 8;  // the largest cluster
 // most four, then enough to keep eight a thread in registers, up to eight
 inline int select_ctas(int n) { return n <= 4 * kSelThreads ? 1 : n <= 16 * kSelThreads ? 4 : kSelCtas; }
 
-// the keys below `key` and `take` of the `equal` ones that equal it are the
-// wanted ones
+// the keys below `key` (which need not be one) and `take` of the `equal` ones
+// that equal it are the wanted ones
 struct Cut {
   uint32_t key;
   int take, equal;
@@ -148,7 +148,9 @@ __device__ __forceinline__ Cut cluster_select(cooperative_groups::cluster_group&
     need -= sh.before;
     equal = sh.in_bin;
     __syncthreads();
-    if (shift == 0) break;  // (the same in every thread of the cluster)
+    // (these are the same in every thread of the cluster)
+    if (shift == 0) break;
+    if (need == equal) return Cut{hi + 1u, 0, 0};  // the whole bin is wanted (usually after two passes)
   }
   return Cut{lo, (int)need, (int)equal};
 }
