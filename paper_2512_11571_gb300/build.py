@@ -20,7 +20,7 @@ BUILD = os.path.join(HERE, "_build")
 # (-DCEM_DEBUG; see cem_debug_status), in its own object folder and library
 DEBUG_OUT = os.path.join(HERE, "libcemtamp_debug.so")
 DEBUG_BUILD = os.path.join(HERE, "_build_debug")
-SOURCES = ["capi.cu", "sample.cu", "rollout.cu", "refit.cu", "batch.cu", "surrogate.cu", "mlp_tc.cu", "gemm_tc.cu", "solve_static.cu"]
+SOURCES = ["capi.cu", "sample.cu", "rollout.cu", "refit.cu", "batch.cu", "surrogate.cu", "mlp_tc.cu", "mlp_train.cu", "gemm_tc.cu", "solve_static.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xptxas", "-O3"]
 

@@ -300,6 +300,60 @@ bool gemm_tc_supported(const GemmArgs& g);
 // pipeline wait that runs out sets *status (device int) non-zero
 cudaError_t gemm_tc(int epi, const GemmArgs& g, int* status, cudaStream_t st);
 
+// ---- fused training step of the 48 -> 4 x 256 -> 1 surrogate (csrc/mlp_train.cu)
+constexpr int kTrainIn = 48, kTrainWidth = 256, kTrainDepth = 4;
+constexpr int kTrainRows = 64;  // rows per CTA; every row buffer holds tiles x 64 rows
+// float4 offset of layer l's partial sums inside a chunk's, and their number
+__host__ __device__ constexpr int train_part4(int l) {
+  return l == 0 ? 0 : (kTrainIn / 4 + (l - 1) * (kTrainWidth / 4)) * kTrainWidth;
+}
+constexpr int kTrainPart4 = train_part4(kTrainDepth);
+struct TrainArgs {
+  // data: FP32 rows x[][48] and targets t[]; the step's rows are drawn from
+  // draw_from of them (Philox on the step), or, if that is 0, the first
+  // `batch` in order and only the gradient is formed (into g)
+  const float* x;
+  const float* t;
+  const float* norm;  // [mu, sigma]
+  int batch, tiles, draw_from;
+  uint64_t seed;
+  int chunk, chunks;  // rows per split-K chunk (a multiple of 32) and their number
+  // parameters: FP32 masters, BF16 copy, weight image (read, and written by
+  // the update), offsets of the layers' weights and biases
+  float* p;
+  __nv_bfloat16* pb;
+  const uint8_t* wpack;
+  uint8_t* wpack_out;
+  const float* bias[kTrainDepth + 1];
+  const __nv_bfloat16* w_out;
+  int w_off[kTrainDepth + 1], b_off[kTrainDepth + 1];
+  // workspace
+  uint8_t* act[kTrainDepth];  // layer inputs and layer gradients, operand images
+  uint8_t* dz[kTrainDepth];
+  float* gprime;              // GELU' [layer][tile][row / 4][feature][4]
+  float* dy;
+  float* sq;                  // squared residuals
+  float* part;                // [chunk][kTrainPart4] float4
+  float* biaspart;            // [chunk][layer][256]
+  float* colpart;             // [tile][256]
+  float* losspart;            // [(batch + 255) / 256]
+  // results
+  float* g;
+  float* m1;
+  float* m2;
+  float* loss_d;  // sum of the squared residuals
+  float* hist;    // per step (may be null)
+  float lr, b1, b2, eps, wd;
+  int* step_d;
+  long long* adam_t_d;
+  int* status;
+};
+bool train_supported(int in_dim, int width, int depth);
+size_t train_pack_bytes();
+// the weight image from pb (before the first step of a call)
+cudaError_t train_pack(const TrainArgs& a, cudaStream_t st);
+cudaError_t train_step(const TrainArgs& a, cudaStream_t st);
+
 // Every device allocation of the library goes through dev_malloc: a plain
 // cudaMalloc, except that the test hook cem_test_fail_allocation can make
 // the k-th next one report cudaErrorMemoryAllocation without allocating

@@ -317,36 +317,59 @@ __global__ void finish_sum_kernel(const float* __restrict__ partial, int n, floa
   if (threadIdx.x == 0) out[0] = red[0];
 }
 
-// mean and standard deviation of t[M] in FP64 (single block, fixed order):
-// norm[0] = mean, norm[1] = std (1 if degenerate)
-__global__ void target_stats_kernel(const float* __restrict__ t, int M, float* __restrict__ norm) {
+// mean and standard deviation of t[M] in FP64 (fixed order): norm[0] = mean,
+// norm[1] = std (1 if degenerate).  A grid of up to kStatBlocks sums runs,
+// every block of the second pass adds the first's sums in order; bound by
+// reading t twice (one block alone: 2.97 ms for 1,048,576 targets).
+constexpr int kStatBlocks = 304;
+
+__device__ __forceinline__ double block_sum_f64(double s, double* red) {
+  red[threadIdx.x] = s;
+  __syncthreads();
+  for (int k = blockDim.x / 2; k > 0; k >>= 1) {
+    if (threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
+    __syncthreads();
+  }
+  const double v = red[0];
+  __syncthreads();
+  return v;
+}
+
+// pass 0: part[b] = sums of t; pass 1: part[kStatBlocks + b] = sums of
+// (t - mean)^2; pass 2 (one block): norm
+__global__ void __launch_bounds__(256) target_stats_kernel(const float* __restrict__ t, int M, int pass, int blocks,
+                                                           double* __restrict__ part, float* __restrict__ norm) {
   __shared__ double red[256];
+  double mean = 0.0;
+  if (pass > 0) {
+    double s = 0.0;
+    for (int i = threadIdx.x; i < blocks; i += 256) s += part[i];
+    mean = block_sum_f64(s, red) / M;
+  }
   double s = 0.0;
-  for (int i = threadIdx.x; i < M; i += blockDim.x) s += t[i];
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int k = blockDim.x / 2; k > 0; k >>= 1) {
-    if (threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
-    __syncthreads();
+  if (pass < 2) {
+    for (long long i = blockIdx.x * 256 + threadIdx.x; i < M; i += blocks * 256) {
+      const double d = (double)t[i] - mean;
+      s += pass == 0 ? (double)t[i] : d * d;
+    }
+    s = block_sum_f64(s, red);
+    if (threadIdx.x == 0) part[pass * kStatBlocks + blockIdx.x] = s;
+    return;
   }
-  const double mean = red[0] / M;
-  __syncthreads();
-  s = 0.0;
-  for (int i = threadIdx.x; i < M; i += blockDim.x) {
-    const double d = t[i] - mean;
-    s += d * d;
-  }
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int k = blockDim.x / 2; k > 0; k >>= 1) {
-    if (threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
-    __syncthreads();
-  }
+  for (int i = threadIdx.x; i < blocks; i += 256) s += part[kStatBlocks + i];
+  s = block_sum_f64(s, red);
   if (threadIdx.x == 0) {
-    const double sd = sqrt(red[0] / M);
+    const double sd = sqrt(s / M);
     norm[0] = (float)mean;
     norm[1] = sd > 1e-12 ? (float)sd : 1.0f;
   }
+}
+
+void target_stats(const float* t, int M, double* part, float* norm, cudaStream_t st) {
+  const int blocks = std::min(kStatBlocks, (M + 1023) / 1024);
+  target_stats_kernel<<<blocks, 256, 0, st>>>(t, M, 0, blocks, part, norm);
+  target_stats_kernel<<<blocks, 256, 0, st>>>(t, M, 1, blocks, part, norm);
+  target_stats_kernel<<<1, 256, 0, st>>>(t, M, 2, blocks, part, norm);
 }
 
 struct Segs {
@@ -374,14 +397,7 @@ __global__ void adamw_kernel(float* __restrict__ p, const float* __restrict__ gr
   int decay = 0;
   for (int s = 0; s < segs.n; ++s)
     if (i >= segs.off[s] && i < segs.off[s] + segs.len[s]) decay = segs.decay[s];
-  const float g = grad[i];
-  const float a = b1 * m1[i] + (1.0f - b1) * g;
-  const float v = b2 * m2[i] + (1.0f - b2) * g * g;
-  m1[i] = a;
-  m2[i] = v;
-  float x = p[i];
-  x = x - lr * (decay ? wd : 0.0f) * x - lr * (a / c1) / (sqrtf(v / c2) + eps);
-  p[i] = x;
+  const float x = adamw(p, m1, m2, i, grad[i], decay, lr, b1, b2, eps, wd, c1, c2);
   pb[i] = __float2bfloat16_rn(x);
 }
 
@@ -790,6 +806,9 @@ struct cem_surrogate_ctx {
   float* loss_d = nullptr;
   float* splitk = nullptr;   // split-K partials of the weight gradients
   float* colpart = nullptr;  // row-chunk partials of the bias gradients
+  // fused training step (csrc/mlp_train.cu): its workspace, one block
+  uint8_t* train_work = nullptr;
+  size_t train_bytes = 0;
   // screening workspace
   int cap_pool = 0;
   float* pool_theta = nullptr;
@@ -800,6 +819,7 @@ struct cem_surrogate_ctx {
   // change), status word of its bounded waits, path selection
   void* tc_pack = nullptr;
   int* tc_status = nullptr;
+  double* stat_part = nullptr;   // partial sums of the target statistics
   int* step_d = nullptr;         // training: step of the current cem_surrogate_train call
   long long* adam_t_d = nullptr;  // training: AdamW steps taken (mirrors adam_step)
   bool tc_pack_valid = false;
@@ -825,6 +845,9 @@ void sur_free_work(cem_surrogate_ctx* s) {
   cudaFree(s->loss_d);
   cudaFree(s->splitk);
   cudaFree(s->colpart);
+  cudaFree(s->train_work);
+  s->train_work = nullptr;
+  s->train_bytes = 0;
   s->splitk = nullptr;
   s->colpart = nullptr;
   s->xin = nullptr;
@@ -903,6 +926,83 @@ bool use_tc_gemm(const cem_surrogate_ctx* s) { return s->gemm_path != 1; }
 
 bool use_tc(const cem_surrogate_ctx* s) {
   return s->fwd_path != 1 && mlp_tc_supported(s->in_dim, s->width, s->depth);
+}
+
+// the fused training step takes this network (gemm paths 0 and 2)
+bool use_fused_train(const cem_surrogate_ctx* s) {
+  return (s->gemm_path == 0 || s->gemm_path == 2) && train_supported(s->in_dim, s->width, s->depth);
+}
+
+// arguments of the fused step for `batch` rows, its workspace laid out in one
+// block (kept for later calls; a larger batch replaces it)
+int train_args(cem_surrogate_ctx* s, const float* x_d, const float* t_d, int batch, TrainArgs* out) {
+  TrainArgs a;
+  std::memset(&a, 0, sizeof(a));
+  a.x = x_d;
+  a.t = t_d;
+  a.norm = s->norm;
+  a.batch = batch;
+  a.tiles = (batch + kTrainRows - 1) / kTrainRows;
+  a.chunk = split_chunk(batch);
+  a.chunks = (batch + a.chunk - 1) / a.chunk;
+  const size_t rows = (size_t)a.tiles * kTrainRows, W = s->width;
+  size_t o = 0;
+  auto take = [&](size_t bytes) {
+    const size_t at = o;
+    o += (bytes + 255) / 256 * 256;
+    return at;
+  };
+  const size_t pack = take(train_pack_bytes());
+  size_t act[kTrainDepth], dz[kTrainDepth];
+  for (int l = 0; l < kTrainDepth; ++l) {
+    act[l] = take(rows * (size_t)(l == 0 ? s->in_dim : s->width) * 2);
+    dz[l] = take(rows * W * 2);
+  }
+  const size_t gp = take(rows * W * 4 * kTrainDepth), dy = take(rows * 4), sq = take(rows * 4);
+  const size_t part = take(sizeof(float) * 4 * (size_t)kTrainPart4 * a.chunks);
+  const size_t bpart = take(sizeof(float) * W * kTrainDepth * a.chunks), cpart = take(sizeof(float) * W * a.tiles);
+  const size_t lpart = take(sizeof(float) * (((size_t)batch + 255) / 256)), loss = take(sizeof(float));
+  if (o > s->train_bytes || !s->train_work) {
+    cudaFree(s->train_work);
+    s->train_work = nullptr;
+    s->train_bytes = 0;
+    if (dev_malloc(&s->train_work, o) != cudaSuccess) {
+      cudaGetLastError();
+      s->train_work = nullptr;
+      return fail(CEM_ERR_NO_MEMORY, "training workspace allocation failed");
+    }
+    s->train_bytes = o;
+  }
+  uint8_t* w = s->train_work;
+  a.p = s->p;
+  a.pb = s->pb;
+  a.wpack = a.wpack_out = w + pack;
+  for (int l = 0; l <= kTrainDepth; ++l) {
+    a.bias[l] = s->p + s->b_off[l];
+    a.w_off[l] = s->w_off[l];
+    a.b_off[l] = s->b_off[l];
+  }
+  a.w_out = s->pb + s->w_off[kTrainDepth];
+  for (int l = 0; l < kTrainDepth; ++l) {
+    a.act[l] = w + act[l];
+    a.dz[l] = w + dz[l];
+  }
+  a.gprime = reinterpret_cast<float*>(w + gp);
+  a.dy = reinterpret_cast<float*>(w + dy);
+  a.sq = reinterpret_cast<float*>(w + sq);
+  a.part = reinterpret_cast<float*>(w + part);
+  a.biaspart = reinterpret_cast<float*>(w + bpart);
+  a.colpart = reinterpret_cast<float*>(w + cpart);
+  a.losspart = reinterpret_cast<float*>(w + lpart);
+  a.loss_d = reinterpret_cast<float*>(w + loss);
+  a.g = s->g;
+  a.m1 = s->m1;
+  a.m2 = s->m2;
+  a.step_d = s->step_d;
+  a.adam_t_d = s->adam_t_d;
+  a.status = s->tc_status;
+  *out = a;
+  return CEM_OK;
 }
 
 // scores of M rows, no activations kept: the fused tcgen05 kernel where the
@@ -1203,6 +1303,7 @@ int cem_surrogate_create(int in_dim, int width, int depth, uint64_t seed, cem_su
   A((void**)&s->norm, sizeof(float) * 2);
   if (mlp_tc_supported(in_dim, width, depth)) A(&s->tc_pack, mlp_tc_pack_bytes());
   A((void**)&s->tc_status, sizeof(int));
+  A((void**)&s->stat_part, sizeof(double) * 2 * kStatBlocks);
   A((void**)&s->step_d, sizeof(int));
   A((void**)&s->adam_t_d, sizeof(long long));
   if (e == cudaSuccess) e = cudaMemset(s->tc_status, 0, sizeof(int));
@@ -1230,7 +1331,7 @@ int cem_surrogate_destroy(cem_surrogate_handle s) {
   sur_free_work(s);
   void* ptrs[] = {s->p, s->pb, s->g, s->m1, s->m2, s->norm,
                   s->pool_theta, s->pool_x, s->pool_score, s->keep_idx, s->tc_pack, s->tc_status,
-                  s->step_d, s->adam_t_d};
+                  s->step_d, s->adam_t_d, s->stat_part};
   for (void* p : ptrs) cudaFree(p);
   delete s;
   return CEM_OK;
@@ -1348,9 +1449,17 @@ int cem_surrogate_gradient(cem_surrogate_handle s, const float* x_d, const float
   if (!s || !grad_h) return fail(CEM_ERR_INVALID_ARG, "null argument");
   if (M < 1 || M > (1 << 22)) return fail(CEM_ERR_UNSUPPORTED, "M must be in 1..2^22");
   if (!is_dev(x_d) || !is_dev(t_d)) return fail(CEM_ERR_INVALID_ARG, "x and t must be device pointers");
+  const float* loss_d = nullptr;  // (s->loss_d where it stays null)
   if (s->gemm_path == 3) {
     int rc = gradient_f32(s, x_d, t_d, M);
     if (rc != CEM_OK) return rc;
+  } else if (use_fused_train(s)) {
+    TrainArgs a;
+    int rc = train_args(s, x_d, t_d, M, &a);
+    if (rc != CEM_OK) return rc;
+    SUR_CUDA(train_pack(a, 0));
+    SUR_CUDA(train_step(a, 0));
+    loss_d = a.loss_d;
   } else {
     int rc = load_features(s, x_d, M, 0);
     if (rc != CEM_OK) return rc;
@@ -1362,7 +1471,7 @@ int cem_surrogate_gradient(cem_surrogate_handle s, const float* x_d, const float
   SUR_CUDA(cudaMemcpy(grad_h, s->g, sizeof(float) * s->total, cudaMemcpyDeviceToHost));
   if (loss_h) {
     float l = 0.0f;
-    SUR_CUDA(cudaMemcpy(&l, s->loss_d, sizeof(float), cudaMemcpyDeviceToHost));
+    SUR_CUDA(cudaMemcpy(&l, loss_d ? loss_d : s->loss_d, sizeof(float), cudaMemcpyDeviceToHost));
     *loss_h = l / M;
   }
   return CEM_OK;
@@ -1374,11 +1483,12 @@ int cem_surrogate_train(cem_surrogate_handle s, const float* x_d, const float* t
   if (M < 1 || batch < 1 || batch > (1 << 20) || steps < 0 || steps > 10000000)
     return fail(CEM_ERR_UNSUPPORTED, "M >= 1, batch in 1..2^20, steps in 0..1e7");
   if (!is_dev(x_d) || !is_dev(t_d)) return fail(CEM_ERR_INVALID_ARG, "x and t must be device pointers");
-  // whole data set in BF16 once
+  const bool fused = use_fused_train(s);
+  // layer-by-layer path: the whole data set in BF16 once (the fused step rounds the rows it draws)
   bf16* Xall = nullptr;
   float* hist_d = nullptr;  // per-step losses stay on the device until the end (no per-step sync)
   cudaStream_t st = nullptr;
-  if (dev_malloc(&Xall, sizeof(bf16) * (size_t)M * s->in_dim) != cudaSuccess ||
+  if ((!fused && dev_malloc(&Xall, sizeof(bf16) * (size_t)M * s->in_dim) != cudaSuccess) ||
       (loss_hist_h && steps > 0 && dev_malloc(&hist_d, sizeof(float) * (size_t)steps) != cudaSuccess)) {
     cudaGetLastError();
     cudaFree(Xall);
@@ -1392,9 +1502,10 @@ int cem_surrogate_train(cem_surrogate_handle s, const float* x_d, const float* t
   }
   cudaDeviceSynchronize();  // earlier work on other streams (parameters, data) is complete
   const size_t n = (size_t)M * s->in_dim;
-  to_bf16_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(x_d, n, Xall);
-  if (normalize) target_stats_kernel<<<1, 256, 0, st>>>(t_d, M, s->norm);
-  int rc = ensure_rows(s, batch);
+  if (!fused) to_bf16_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(x_d, n, Xall);
+  if (normalize) target_stats(t_d, M, s->stat_part, s->norm, st);
+  TrainArgs ta;
+  int rc = fused ? train_args(s, x_d, t_d, batch, &ta) : ensure_rows(s, batch);
   if (rc != CEM_OK) {
     cudaStreamDestroy(st);
     cudaFree(Xall);
@@ -1421,14 +1532,26 @@ int cem_surrogate_train(cem_surrogate_handle s, const float* x_d, const float* t
     step_end_kernel<<<1, 1, 0, st>>>(s->step_d, s->adam_t_d, s->loss_d, hist_d);
     return cudaGetLastError();
   };
+  int done = 0;
+  if (fused && e == cudaSuccess && steps > 0) {  // three launches a step, shorter to issue than to run
+    ta.draw_from = M;
+    ta.seed = seed;
+    ta.hist = hist_d;
+    ta.lr = lr;
+    ta.b1 = b1;
+    ta.b2 = b2;
+    ta.eps = eps;
+    ta.wd = weight_decay;
+    e = train_pack(ta, st);
+    for (; done < steps && e == cudaSuccess; ++done) e = train_step(ta, st);
+  }
   // the first step runs directly (it also sets up the kernels), the others
   // replay that step captured as one CUDA graph; direct launches if capture fails
-  int done = 0;
-  if (e == cudaSuccess && steps > 0) {
+  if (e == cudaSuccess && done < steps) {
     e = enqueue_step();
     done = 1;
   }
-  if (e == cudaSuccess && steps > 1) {
+  if (e == cudaSuccess && done < steps) {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
