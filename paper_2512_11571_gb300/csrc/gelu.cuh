@@ -19,16 +19,26 @@ __device__ __forceinline__ void gelu_both(float z, float& act, float& grad) {
   grad = gelu_grad(z);
 }
 
-// one AdamW update of parameter i (decoupled decay), moments included; c1, c2
-// the bias corrections 1 - b^t.  Returns the new parameter.
+// one AdamW update (decoupled decay) of a parameter x and its moments by the
+// gradient g; c1, c2: the bias corrections 1 - b^t.  The roundings are written
+// out: training follows every last bit of its first steps.
+__device__ __forceinline__ void adamw_value(float& x, float& m1, float& m2, float g, int decay, float lr, float b1, float b2,
+                                            float eps, float wd, float c1, float c2) {
+  const float a = __fmaf_rn(1.0f - b1, g, __fmul_rn(b1, m1));
+  const float v = __fmaf_rn(__fmul_rn(1.0f - b2, g), g, __fmul_rn(b2, m2));
+  m1 = a;
+  m2 = v;
+  const float kept = __fmaf_rn(-__fmul_rn(lr, decay ? wd : 0.0f), x, x);
+  x = __fsub_rn(kept, __fmul_rn(lr, a / c1) / (sqrtf(v / c2) + eps));
+}
+
+// the same on parameter i in memory; returns the new parameter
 __device__ __forceinline__ float adamw(float* __restrict__ p, float* __restrict__ m1, float* __restrict__ m2, int i, float g,
                                        int decay, float lr, float b1, float b2, float eps, float wd, float c1, float c2) {
-  const float a = b1 * m1[i] + (1.0f - b1) * g;
-  const float v = b2 * m2[i] + (1.0f - b2) * g * g;
+  float x = p[i], a = m1[i], v = m2[i];
+  adamw_value(x, a, v, g, decay, lr, b1, b2, eps, wd, c1, c2);
   m1[i] = a;
   m2[i] = v;
-  float x = p[i];
-  x = x - lr * (decay ? wd : 0.0f) * x - lr * (a / c1) / (sqrtf(v / c2) + eps);
   p[i] = x;
   return x;
 }

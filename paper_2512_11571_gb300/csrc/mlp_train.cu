@@ -154,6 +154,20 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
 #pragma unroll
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+// Programmatic dependent launch: the launches of a step overlap their set-up
+// (barriers, TMEM, launch latency); a kernel touches what the one before it
+// wrote or read only after grid_wait, which returns when that one is complete.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&h);
@@ -212,6 +226,8 @@ __global__ void __launch_bounds__(THREADS, 1) train_rows_kernel(const TrainArgs 
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
+  grid_next();
+  grid_wait();
 
   if (warp == EWARPS) {
     // ---- copies and MMAs: layers 0..3 forward, 3..1 backward, one lane ----
@@ -333,7 +349,6 @@ __global__ void __launch_bounds__(THREADS, 1) train_rows_kernel(const TrainArgs 
     };
     uint32_t nacc = 0;
     bool ok = true;
-    float v[32];
     for (int l = 0; l < DEPTH; ++l) {
       if (ok && !mbar_wait(accb + 8 * half, nacc & 1u, &s_fail, 2 * kWaitLimitNs)) {
         ok = false;
@@ -343,21 +358,22 @@ __global__ void __launch_bounds__(THREADS, 1) train_rows_kernel(const TrainArgs 
       ++nacc;
       if (ok) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        tmem_ld32(tacc, v);
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         const float b = sbias[l * W + f];
         uint8_t* out = sm + SM_A + (uint32_t)(l & 1) * image_bytes(R, W);
+        // eight rows at a time, not unrolled: 32 copies of the erf and the
+        // exponential outgrew the instruction cache (1.8 of 11.4 stall cycles)
+#pragma unroll 1
+        for (int q = 0; q < 4; ++q) {
+          float v[8], g[8];
+          tmem_ld8(tacc + 8u * (uint32_t)q, v);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {  // eight rows
-          float g[8];
-#pragma unroll
-          for (int i = 0; i < 8; ++i) gelu_both(v[8 * q + i] + b, v[8 * q + i], g[i]);
+          for (int i = 0; i < 8; ++i) gelu_both(v[i] + b, v[i], g[i]);
           *gprime(l, 2 * q) = make_float4(g[0], g[1], g[2], g[3]);
           *gprime(l, 2 * q + 1) = make_float4(g[4], g[5], g[6], g[7]);
           *reinterpret_cast<uint4*>(out + image_off(grp * 32 + 8 * q, f, W)) =
-              make_uint4(pack2(v[8 * q], v[8 * q + 1]), pack2(v[8 * q + 2], v[8 * q + 3]), pack2(v[8 * q + 4], v[8 * q + 5]),
-                         pack2(v[8 * q + 6], v[8 * q + 7]));
+              make_uint4(pack2(v[0], v[1]), pack2(v[2], v[3]), pack2(v[4], v[5]), pack2(v[6], v[7]));
         }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       }
       if (l + 1 < DEPTH) {
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -409,32 +425,36 @@ __global__ void __launch_bounds__(THREADS, 1) train_rows_kernel(const TrainArgs 
     }
     // dz_3 = dy w_out GELU'(z_3), then dz_{l-1} = (dz_l W_l) GELU'(z_{l-1})
     for (int l = DEPTH - 1; l >= 0; --l) {
-      if (l == DEPTH - 1) {
-        const float w = swout[f];
+      float4 g[8];  // GELU' is on its way while the product runs
 #pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] = sdy[grp * 32 + i] * w;
-      } else {
+      for (int q = 0; q < 8; ++q) g[q] = *gprime(l, q);
+      if (l < DEPTH - 1) {
         if (ok && !mbar_wait(accb + 8 * half, nacc & 1u, &s_fail, 2 * kWaitLimitNs)) {
           ok = false;
           if (!s_fail) s_fail = 9;
         }
         ok = __all_sync(0xffffffffu, ok);
         ++nacc;
-        if (ok) {
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          tmem_ld32(tacc, v);
-          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        }
+        if (ok) asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       }
       if (ok) {
         uint8_t* out = sm + SM_A + (uint32_t)(l & 1 ? 0 : 1) * image_bytes(R, W);
+        const float w = swout[f];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          const float4 g0 = *gprime(l, 2 * q), g1 = *gprime(l, 2 * q + 1);
+          float v[8];
+          if (l < DEPTH - 1) {
+            tmem_ld8(tacc + 8u * (uint32_t)q, v);
+          } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = sdy[grp * 32 + 8 * q + i] * w;
+          }
+          const float4 g0 = g[2 * q], g1 = g[2 * q + 1];
           *reinterpret_cast<uint4*>(out + image_off(grp * 32 + 8 * q, f, W)) =
-              make_uint4(pack2(v[8 * q] * g0.x, v[8 * q + 1] * g0.y), pack2(v[8 * q + 2] * g0.z, v[8 * q + 3] * g0.w),
-                         pack2(v[8 * q + 4] * g1.x, v[8 * q + 5] * g1.y), pack2(v[8 * q + 6] * g1.z, v[8 * q + 7] * g1.w));
+              make_uint4(pack2(v[0] * g0.x, v[1] * g0.y), pack2(v[2] * g0.z, v[3] * g0.w), pack2(v[4] * g1.x, v[5] * g1.y),
+                         pack2(v[6] * g1.z, v[7] * g1.w));
         }
+        if (l < DEPTH - 1) asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
@@ -449,24 +469,38 @@ __global__ void __launch_bounds__(THREADS, 1) train_rows_kernel(const TrainArgs 
 }
 
 // ---------------------------------------------------------------- weights
+// A CTA takes 128 outputs x 128 inputs (layer 0: all 48) of one chunk: rounds
+// of 64 rows through a ring of three, so that the copies run ahead of the
+// MMAs, and two CTAs an SM (104 KB, 256 TMEM columns each), so that one's
+// stores run beside the other's copies.  (Whole chunks of 256 rows and 256
+// inputs, one CTA an SM, copied, multiplied and stored in turn: 17.4 us.)
+// Bound by the partial sums' stores and the update's loads of them (26 MB
+// each way through L2 at 8192 rows).
 constexpr int BTHREADS = 256;  // epilogue: warp w drains lane quadrant w % 4, half w / 4 of the columns
-constexpr int KSUB = 256;      // rows in shared memory at a time
-constexpr uint32_t SB_A = 0;                                   // dz^T, 128 outputs x 256 rows
-constexpr uint32_t SB_B = SB_A + image_bytes(KSUB, 128);       // a^T, 256 inputs x 256 rows
-constexpr uint32_t SB_ONE = SB_B + image_bytes(KSUB, W);       // 16 x 256: a row of ones (the bias gradient)
-constexpr uint32_t SB_BAR = SB_ONE + image_bytes(16, KSUB);    // copies, MMAs of a round, all MMAs
-constexpr uint32_t SB_TMEM = SB_BAR + 24;
+constexpr int KSUB = 64;       // rows per round
+constexpr int BSTAGES = 3;
+constexpr int BN = 128;        // inputs per CTA
+constexpr uint32_t kStageA = image_bytes(KSUB, 128), kStageB = image_bytes(KSUB, BN), kStage = kStageA + kStageB;
+constexpr uint32_t SB_ONE = BSTAGES * kStage;                  // 16 x 64: a row of ones (the bias gradient)
+constexpr uint32_t SB_BAR = SB_ONE + image_bytes(16, KSUB);    // per stage: copied, read; all MMAs done
+constexpr uint32_t SB_TMEM = SB_BAR + (2 * BSTAGES + 1) * 8;
 constexpr uint32_t SB_TOTAL = SB_TMEM + 16;
-static_assert(SB_TOTAL + 1024 + 64 <= 227 * 1024, "shared memory plan exceeds 227 KB");
+static_assert(2 * (SB_TOTAL + 2048 + 1024) <= 227 * 1024, "two CTAs per SM");
+constexpr uint32_t kColsB = 256;  // TMEM columns: 128 of the product, 16 of the bias at kColBias
+constexpr uint32_t kColBias = 128;
+// CTAs per chunk: layers 1 to 3 in four tiles, layer 0 in two
+constexpr int kTiles = 4 * (DEPTH - 1) + 2;
 
-__global__ void __launch_bounds__(BTHREADS, 1) train_weights_kernel(const TrainArgs a) {
+__global__ void __launch_bounds__(BTHREADS, 2) train_weights_kernel(const TrainArgs a) {
   extern __shared__ __align__(1024) uint8_t sm[];
   __shared__ volatile int s_fail;
   __shared__ float red[256];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if ((int)blockIdx.x >= 2 * DEPTH * a.chunks) {
+  if ((int)blockIdx.x >= kTiles * a.chunks) {
+    grid_next();
+    grid_wait();
     // squared residuals of 256 rows, and the step counters (nothing of this launch reads them)
-    const int b = (int)blockIdx.x - 2 * DEPTH * a.chunks, i = b * 256 + tid;
+    const int b = (int)blockIdx.x - kTiles * a.chunks, i = b * 256 + tid;
     red[tid] = i < a.batch ? a.sq[i] : 0.0f;
     __syncthreads();
     for (int s = 128; s > 0; s >>= 1) {
@@ -482,68 +516,86 @@ __global__ void __launch_bounds__(BTHREADS, 1) train_weights_kernel(const TrainA
     }
     return;
   }
-  const int l = DEPTH - 1 - (int)blockIdx.x / (2 * a.chunks);  // (the small first layer last)
-  const int z = (int)blockIdx.x % (2 * a.chunks) >> 1, half = (int)blockIdx.x & 1;
-  const int K = l == 0 ? IN : W;
+  // (the small first layer last)
+  const int z = (int)blockIdx.x % a.chunks, piece = (int)blockIdx.x / a.chunks;
+  const int l = piece < 4 * (DEPTH - 1) ? DEPTH - 1 - piece / 4 : 0;
+  const int half = piece & 1, side = l == 0 ? 0 : (piece >> 1) & 1;  // outputs 128 half .., inputs 128 side ..
+  const int N = l == 0 ? IN : BN;
   const int rbeg = z * a.chunk, rend = min(a.tiles * R, rbeg + a.chunk);
-  const uint32_t base = smem_u32(sm), inb = base + SB_BAR, mmab = inb + 8, doneb = inb + 16;
+  const uint32_t base = smem_u32(sm), fullb = base + SB_BAR, freeb = fullb + 8 * BSTAGES, doneb = freeb + 8 * BSTAGES;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + SB_TMEM);
   if (tid == 0) {
     s_fail = 0;
-    mbar_init(inb, 1);
-    mbar_init(mmab, 1);
+    for (int i = 0; i < BSTAGES; ++i) {
+      mbar_init(fullb + 8 * i, 1);
+      mbar_init(freeb + 8 * i, 1);
+    }
     mbar_init(doneb, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  // ones operand, K-major: core (n / 8, k / 8) at ((n / 8) 32 + k / 8) 128
-  for (int i = tid; i < 2 * 32 * 8; i += BTHREADS) {
-    const int nb = i >> 8, kb = (i >> 3) & 31, n = i & 7;
+  // ones operand, K-major: core (n / 8, k / 8) at ((n / 8) 8 + k / 8) 128
+  for (int i = tid; i < 2 * (KSUB / 8) * 8; i += BTHREADS) {
+    const int nb = i / (KSUB / 8 * 8), kb = (i >> 3) % (KSUB / 8), n = i & 7;
     const uint32_t one = nb == 0 && n == 0 ? 0x3F803F80u : 0u;
-    *reinterpret_cast<uint4*>(sm + SB_ONE + (uint32_t)(nb * 32 + kb) * 128u + (uint32_t)n * 16u) = make_uint4(one, one, one, one);
+    *reinterpret_cast<uint4*>(sm + SB_ONE + (uint32_t)(nb * (KSUB / 8) + kb) * 128u + (uint32_t)n * 16u) = make_uint4(one, one, one, one);
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   __syncwarp();
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512u));
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(kColsB));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
-  const int nsub = rend > rbeg ? (rend - rbeg + KSUB - 1) / KSUB : 0;
+  grid_next();
+  grid_wait();
+  const int nsub = (rend - rbeg + KSUB - 1) / KSUB;
   if (tid == 0) {
-    const uint32_t idesc = make_idesc(K, 0, 0), idesc1 = make_idesc(16, 0, 0);
-    bool copying = false, pending = false;
-    uint32_t phase = 0;  // of the round in progress
-    for (int sub = 0; sub < nsub; ++sub) {
-      const int r0 = rbeg + sub * KSUB, rows = min(KSUB, rend - r0), groups = rows >> 3;
-      // the last round's MMAs have read the operands
-      if (sub > 0 && !mbar_wait(mmab, (uint32_t)(sub - 1) & 1u, &s_fail)) { s_fail = 11; break; }
-      pending = false;
-      phase = (uint32_t)sub & 1u;
-      expect(inb, image_bytes(rows, 128) + image_bytes(rows, K));
-      copying = true;
+    const uint32_t idesc = make_idesc(N, 0, 0), idesc1 = make_idesc(16, 0, 0);
+    int issued = 0;  // rounds whose copies were issued
+    int used = 0;    // rounds whose MMAs were issued
+    auto copy = [&](int i) {
+      const int r0 = rbeg + i * KSUB, rows = min(KSUB, rend - r0), groups = rows >> 3;
+      const uint32_t st = base + (uint32_t)(i % BSTAGES) * kStage, bar = fullb + 8 * (i % BSTAGES);
+      expect(bar, image_bytes(rows, 128) + image_bytes(rows, N));
       for (int g = 0; g < groups; ++g)
-        bulk_in(base + SB_A + (uint32_t)g * 2048u, a.dz[l] + ((size_t)(r0 >> 3) + g) * (W / 8) * 128 + (size_t)half * 2048, 2048u, inb);
-      bulk_in(base + SB_B, a.act[l] + (size_t)(r0 >> 3) * (K / 8) * 128, image_bytes(rows, K), inb);
-      if (!mbar_wait(inb, (uint32_t)sub & 1u, &s_fail)) { s_fail = 12; break; }
-      copying = false;
+        bulk_in(st + (uint32_t)g * 2048u, a.dz[l] + ((size_t)(r0 >> 3) + g) * (W / 8) * 128 + (size_t)half * 2048, 2048u, bar);
+      if (l == 0)
+        bulk_in(st + kStageA, a.act[0] + (size_t)(r0 >> 3) * (IN / 8) * 128, image_bytes(rows, IN), bar);
+      else
+        for (int g = 0; g < groups; ++g)
+          bulk_in(st + kStageA + (uint32_t)g * 2048u, a.act[l] + ((size_t)(r0 >> 3) + g) * (W / 8) * 128 + (size_t)side * 2048, 2048u,
+                  bar);
+    };
+    for (; issued < nsub && issued < BSTAGES; ++issued) copy(issued);
+    for (; used < nsub; ++used) {
+      const int sl = used % BSTAGES, rows = min(KSUB, rend - rbeg - used * KSUB);
+      if (!mbar_wait(fullb + 8 * sl, (uint32_t)(used / BSTAGES) & 1u, &s_fail)) { s_fail = 12; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint64_t da = make_desc(base + SB_A, 2048u, 128u), db = make_desc(base + SB_B, (uint32_t)(K >> 3) * 128u, 128u);
-      const uint64_t d1 = make_desc(base + SB_ONE, 128u, 32u * 128u);
+      const uint32_t st = base + (uint32_t)sl * kStage, kb = l == 0 ? (uint32_t)(IN / 8) * 128u : 2048u;
+      const uint64_t da = make_desc(st, 2048u, 128u), db = make_desc(st + kStageA, kb, 128u);
+      const uint64_t d1 = make_desc(base + SB_ONE, 128u, (uint32_t)(KSUB / 8) * 128u);
       for (int k = 0; k < rows; k += 16) {
-        const uint32_t acc = sub > 0 || k > 0 ? 1u : 0u;
+        const uint32_t acc = used > 0 || k > 0 ? 1u : 0u;
         const uint64_t ka = da + (uint64_t)(k >> 3) * 128u;
-        mma(tmem, ka, db + (uint64_t)(k >> 3) * (uint64_t)((K >> 3) * 8), idesc, acc);
-        mma(tmem + 256u, ka, d1 + (uint64_t)(k >> 3) * 8u, idesc1, acc);
+        mma(tmem, ka, db + (uint64_t)(k >> 3) * (uint64_t)(kb >> 4), idesc, acc);
+        if (side == 0) mma(tmem + kColBias, ka, d1 + (uint64_t)(k >> 3) * 8u, idesc1, acc);
       }
-      commit(mmab);
-      pending = true;
+      commit(freeb + 8 * sl);
+      if (issued < nsub) {  // the next copies take the stage of the round before, once its MMAs have read it
+        const int prev = issued - BSTAGES;
+        if (prev < used) {
+          if (!mbar_wait(freeb + 8 * (prev % BSTAGES), (uint32_t)(prev / BSTAGES) & 1u, &s_fail)) { ++used; s_fail = 11; break; }
+          copy(issued);
+          ++issued;
+        }
+      }
     }
     if (s_fail) {  // (bounded) what is in flight lands first
-      if (copying) mbar_wait(inb, phase, nullptr);
-      if (pending) mbar_wait(mmab, phase, nullptr);
+      for (int i = used; i < issued; ++i) mbar_wait(fullb + 8 * (i % BSTAGES), (uint32_t)(i / BSTAGES) & 1u, nullptr);
+      if (used > 0) mbar_wait(freeb + 8 * ((used - 1) % BSTAGES), (uint32_t)((used - 1) / BSTAGES) & 1u, nullptr);
     } else {
       commit(doneb);
     }
@@ -559,20 +611,21 @@ __global__ void __launch_bounds__(BTHREADS, 1) train_weights_kernel(const TrainA
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     // partial sums [chunk][layer][input / 4][output] (float4), biases [chunk][layer][output]
     const int quad = warp & 3, o = half * 128 + quad * 32 + lane;
-    float4* part = reinterpret_cast<float4*>(a.part) + (size_t)z * kTrainPart4 + train_part4(l);
+    float4* part = reinterpret_cast<float4*>(a.part) + (size_t)z * kTrainPart4 + train_part4(l) + (size_t)side * (BN / 4) * W;
     const uint32_t t0 = tmem + ((uint32_t)(quad * 32) << 16);
-    const int cols = K <= 64 ? K : K / 2, c0 = K <= 64 ? 0 : (warp >> 2) * cols;
     float v[32];
-    if (K > 64 || warp < 4)
-      for (int c = c0; c < c0 + cols; c += 32) {
-        tmem_ld32(t0 + (uint32_t)c, v);  // (layer 0: columns 48 .. 63 hold nothing and are not stored)
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-          if (c + 4 * q < K) part[(size_t)(c / 4 + q) * W + o] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-      }
-    if (warp >= 4) {
+    for (int i = 0; i < 2; ++i) {
+      const int c = (warp >> 2) * (l == 0 ? 32 : 64) + 32 * i;
+      if (l == 0 && i > 0) break;
+      tmem_ld32(t0 + (uint32_t)c, v);  // (layer 0: columns 48 .. 63 hold nothing and are not stored)
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        if (c + 4 * q < N) part[(size_t)(c / 4 + q) * W + o] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    }
+    if (side == 0 && warp >= 4) {
       uint32_t b;
-      asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(b) : "r"(t0 + 256u));
+      asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(b) : "r"(t0 + kColBias));
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
       a.biaspart[((size_t)z * DEPTH + l) * W + o] = __uint_as_float(b);
     }
@@ -581,7 +634,7 @@ __global__ void __launch_bounds__(BTHREADS, 1) train_weights_kernel(const TrainA
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (s_fail && tid == 0) atomicExch(a.status, s_fail);
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u));
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kColsB));
 }
 
 // ----------------------------------------------------------------- update
@@ -598,12 +651,14 @@ __global__ void __launch_bounds__(CTHREADS) train_update_kernel(const TrainArgs 
   __shared__ float s_c[2];
   const int tid = threadIdx.x, b = (int)blockIdx.x;
   const bool step = a.draw_from > 0;  // else the gradient alone
+  grid_next();
+  grid_wait();
   if (tid == 0 && step) {
     const float t = (float)*a.adam_t_d;  // (counted by this step's weight launch)
     s_c[0] = 1.0f - powf(a.b1, t);
     s_c[1] = 1.0f - powf(a.b2, t);
   }
-  __syncthreads();
+  if (b >= kUpdate4) __syncthreads();
   auto apply = [&](int i, float g, int decay) -> float {  // returns the new parameter
     if (!step) {
       a.g[i] = g;
@@ -616,9 +671,16 @@ __global__ void __launch_bounds__(CTHREADS) train_update_kernel(const TrainArgs 
     int l = DEPTH - 1;
     while (u < train_part4(l)) --l;
     const int K = l == 0 ? IN : W, q = (u - train_part4(l)) / W, o = (u - train_part4(l)) % W;
+    const int i = a.w_off[l] + o * K + 4 * q;
     const float4* src = reinterpret_cast<const float4*>(a.part) + u;
     float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-#pragma unroll 8
+    float4 p = s, m1 = s, m2 = s;
+    if (step) {  // in flight with the partial sums
+      p = *reinterpret_cast<const float4*>(a.p + i);
+      m1 = *reinterpret_cast<const float4*>(a.m1 + i);
+      m2 = *reinterpret_cast<const float4*>(a.m2 + i);
+    }
+#pragma unroll 16
     for (int z = 0; z < a.chunks; ++z) {
       const float4 v = src[(size_t)z * kTrainPart4];
       s.x += v.x;
@@ -626,13 +688,22 @@ __global__ void __launch_bounds__(CTHREADS) train_update_kernel(const TrainArgs 
       s.z += v.z;
       s.w += v.w;
     }
-    const int i = a.w_off[l] + o * K + 4 * q;
-    const float x0 = apply(i, s.x, 1), x1 = apply(i + 1, s.y, 1), x2 = apply(i + 2, s.z, 1), x3 = apply(i + 3, s.w, 1);
-    if (step) {
-      const uint2 h = make_uint2(pack2(x0, x1), pack2(x2, x3));
-      *reinterpret_cast<uint2*>(a.pb + i) = h;
-      *reinterpret_cast<uint2*>(a.wpack_out + weight_base(l) + weight_off(o, 4 * q, K)) = h;
+    if (!step) {
+      *reinterpret_cast<float4*>(a.g + i) = s;
+      return;
     }
+    __syncthreads();  // the bias corrections
+    const float c1 = s_c[0], c2 = s_c[1];
+    adamw_value(p.x, m1.x, m2.x, s.x, 1, a.lr, a.b1, a.b2, a.eps, a.wd, c1, c2);
+    adamw_value(p.y, m1.y, m2.y, s.y, 1, a.lr, a.b1, a.b2, a.eps, a.wd, c1, c2);
+    adamw_value(p.z, m1.z, m2.z, s.z, 1, a.lr, a.b1, a.b2, a.eps, a.wd, c1, c2);
+    adamw_value(p.w, m1.w, m2.w, s.w, 1, a.lr, a.b1, a.b2, a.eps, a.wd, c1, c2);
+    *reinterpret_cast<float4*>(a.p + i) = p;
+    *reinterpret_cast<float4*>(a.m1 + i) = m1;
+    *reinterpret_cast<float4*>(a.m2 + i) = m2;
+    const uint2 h = make_uint2(pack2(p.x, p.y), pack2(p.z, p.w));
+    *reinterpret_cast<uint2*>(a.pb + i) = h;
+    *reinterpret_cast<uint2*>(a.wpack_out + weight_base(l) + weight_off(o, 4 * q, K)) = h;
     return;
   }
   if (b < kUpdate4 + DEPTH) {
@@ -719,10 +790,23 @@ cudaError_t train_step(const TrainArgs& a, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     configured[dev].store(true, std::memory_order_release);
   }
-  train_rows_kernel<<<a.tiles, THREADS, SM_ROWS, st>>>(a);
-  train_weights_kernel<<<2 * DEPTH * a.chunks + (a.batch + 255) / 256, BTHREADS, SB_TOTAL, st>>>(a);
-  train_update_kernel<<<kUpdate4 + DEPTH + W / 32 + 1, CTHREADS, 0, st>>>(a);
-  return cudaGetLastError();
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  auto launch = [&](void (*kernel)(const TrainArgs), int grid, int threads, size_t smem) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, a);
+  };
+  e = launch(train_rows_kernel, a.tiles, THREADS, SM_ROWS);
+  if (e == cudaSuccess) e = launch(train_weights_kernel, kTiles * a.chunks + (a.batch + 255) / 256, BTHREADS, SB_TOTAL);
+  if (e == cudaSuccess) e = launch(train_update_kernel, kUpdate4 + DEPTH + W / 32 + 1, CTHREADS, 0);
+  return e;
 }
 
 }  // namespace cem
