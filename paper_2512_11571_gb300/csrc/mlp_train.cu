@@ -23,12 +23,13 @@
 // MMAs of a layer take 1,000 cycles and the weights (64 KB halves by bulk
 // copies, the next layer's while this one's epilogue runs) hide behind it.
 //
-// Operand images.  Rows come in groups of eight: core matrix (row / 8,
-// feature / 8) is 8 features x 8 rows, feature f % 8 in 16 bytes of eight
-// rows, at ((row / 8) (F / 8) + feature / 8) 128.  The same bytes are the
-// MN-major B operand of the forward and backward products (N = rows) and the
-// K-major operands of dW (K = rows), and any range of whole groups is
-// contiguous.  Likewise one weight image, core (out / 8, in / 8) of 8 outputs
+// Operand images.  A tile's 64 rows x 256 features are two halves of 128
+// features (the input's 48 are one piece); rows come in groups of eight: core
+// matrix (row / 8, feature / 8) of a half is 8 features x 8 rows, feature
+// f % 8 in 16 bytes of eight rows, at ((row / 8) 16 + feature / 8) 128.  The
+// same bytes are the MN-major B operand of the forward and backward products
+// (N = rows) and the K-major operands of dW (K = rows), and any range of whole
+// groups of a half is contiguous, one bulk copy.  Likewise one weight image, core (out / 8, in / 8) of 8 outputs
 // x 16 bytes of eight inputs, is the K-major A operand of the forward and the
 // MN-major one of the backward product.
 //
@@ -59,9 +60,13 @@ constexpr int R = kTrainRows;                 // rows per CTA
 constexpr uint64_t kWaitLimitNs = 1000000000ull;
 
 __host__ __device__ constexpr uint32_t image_bytes(int rows, int F) { return (uint32_t)rows * (uint32_t)F * 2u; }
-// byte offset of element (r, f) of a [rows x F] image
+// features of a piece of an image with F of them, and its bytes per group of eight rows
+__host__ __device__ constexpr int piece_of(int F) { return F > 128 ? 128 : F; }
+__host__ __device__ constexpr uint32_t group_bytes(int F) { return (uint32_t)piece_of(F) * 16u; }
+// byte offset of element (r, f) of a tile's image with F features
 __host__ __device__ constexpr uint32_t image_off(int r, int f, int F) {
-  return ((uint32_t)(r >> 3) * (uint32_t)(F >> 3) + (uint32_t)(f >> 3)) * 128u + (uint32_t)(f & 7) * 16u + (uint32_t)(r & 7) * 2u;
+  return (uint32_t)(f / piece_of(F)) * image_bytes(R, piece_of(F)) + (uint32_t)(r >> 3) * group_bytes(F) +
+         (uint32_t)((f % piece_of(F)) >> 3) * 128u + (uint32_t)(f & 7) * 16u + (uint32_t)(r & 7) * 2u;
 }
 // byte offset of weight (o, i) of a [256 x K] weight image
 __host__ __device__ constexpr uint32_t weight_off(int o, int i, int K) {
@@ -259,9 +264,9 @@ __global__ void __launch_bounds__(THREADS, 1) train_rows_kernel(const TrainArgs 
         for (int h = 0; h < 2; ++h) {
           if ((l > 0 || h == 0) && !wait_half(h)) { fail = 2; break; }
           const uint32_t wa = base + SM_W + (uint32_t)h * (l == 0 ? kW0Bytes / 2 : kHalf);
-          const uint64_t da = make_desc(wa, 128u, (uint32_t)(K >> 3) * 128u), db = make_desc(in, 128u, (uint32_t)(K >> 3) * 128u);
+          const uint64_t da = make_desc(wa, 128u, (uint32_t)(K >> 3) * 128u), db = make_desc(in, 128u, group_bytes(K));
           for (int k = 0; k < K; k += 16)
-            mma(tmem + (uint32_t)(h * R), da + (uint64_t)(k >> 3) * 8u, db + (uint64_t)(k >> 3) * 8u, idesc, k > 0 ? 1u : 0u);
+            mma(tmem + (uint32_t)(h * R), da + (uint64_t)(k >> 3) * 8u, db + (uint64_t)(image_off(0, k, K) >> 4), idesc, k > 0 ? 1u : 0u);
           // the second half's completion also says that the image copied out above has been read: the
           // epilogue two layers on (one on, at the turn) writes its buffer
           if (h == 1) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
@@ -284,11 +289,11 @@ __global__ void __launch_bounds__(THREADS, 1) train_rows_kernel(const TrainArgs 
         bulk_out(a.dz[l] + (size_t)row0 * W * 2, in, image_bytes(R, W));
         if (l < DEPTH - 1 && !(wait_half(0) && wait_half(1))) { fail = 5; break; }
         const uint32_t idesc = make_idesc(R, 1, 1);
-        const uint64_t db = make_desc(in, 128u, (uint32_t)(W >> 3) * 128u);
+        const uint64_t db = make_desc(in, 128u, group_bytes(W));
         for (int h = 0; h < 2; ++h) {  // inputs 128 h ..
           const uint64_t da = make_desc(base + SM_W + (uint32_t)h * 2048u, (uint32_t)(W >> 3) * 128u, 128u);
           for (int k = 0; k < W; k += 16)
-            mma(tmem + (uint32_t)(h * R), da + (uint64_t)(k >> 3) * (uint64_t)((W >> 3) * 8), db + (uint64_t)(k >> 3) * 8u, idesc,
+            mma(tmem + (uint32_t)(h * R), da + (uint64_t)(k >> 3) * (uint64_t)((W >> 3) * 8), db + (uint64_t)(image_off(0, k, W) >> 4), idesc,
                 k > 0 ? 1u : 0u);
           if (h == 1) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
           commit(accb + 8 * h);
@@ -477,7 +482,7 @@ __global__ void __launch_bounds__(THREADS, 1) train_rows_kernel(const TrainArgs 
 // Bound by the partial sums' stores and the update's loads of them (26 MB
 // each way through L2 at 8192 rows).
 constexpr int BTHREADS = 256;  // epilogue: warp w drains lane quadrant w % 4, half w / 4 of the columns
-constexpr int KSUB = 64;       // rows per round
+constexpr int KSUB = R;        // rows per round, at most
 constexpr int BSTAGES = 3;
 constexpr int BN = 128;        // inputs per CTA
 constexpr uint32_t kStageA = image_bytes(KSUB, 128), kStageB = image_bytes(KSUB, BN), kStage = kStageA + kStageB;
@@ -551,30 +556,32 @@ __global__ void __launch_bounds__(BTHREADS, 2) train_weights_kernel(const TrainA
   const uint32_t tmem = *tmem_slot;
   grid_next();
   grid_wait();
-  const int nsub = (rend - rbeg + KSUB - 1) / KSUB;
+  // rounds: the parts of the chunk in each tile (chunks are multiples of 32 rows)
+  const int tile0 = rbeg / R, nsub = (rend - 1) / R - tile0 + 1;
   if (tid == 0) {
     const uint32_t idesc = make_idesc(N, 0, 0), idesc1 = make_idesc(16, 0, 0);
     int issued = 0;  // rounds whose copies were issued
     int used = 0;    // rounds whose MMAs were issued
+    auto first = [&](int i) { return max(rbeg, (tile0 + i) * R); };
+    auto rows_of = [&](int i) { return min(rend, (tile0 + i + 1) * R) - first(i); };
     auto copy = [&](int i) {
-      const int r0 = rbeg + i * KSUB, rows = min(KSUB, rend - r0), groups = rows >> 3;
+      const uint32_t off = (uint32_t)(first(i) % R) >> 3, rows = (uint32_t)rows_of(i);
       const uint32_t st = base + (uint32_t)(i % BSTAGES) * kStage, bar = fullb + 8 * (i % BSTAGES);
       expect(bar, image_bytes(rows, 128) + image_bytes(rows, N));
-      for (int g = 0; g < groups; ++g)
-        bulk_in(st + (uint32_t)g * 2048u, a.dz[l] + ((size_t)(r0 >> 3) + g) * (W / 8) * 128 + (size_t)half * 2048, 2048u, bar);
+      bulk_in(st, a.dz[l] + (size_t)(tile0 + i) * image_bytes(R, W) + (size_t)half * image_bytes(R, 128) + off * group_bytes(W),
+              image_bytes(rows, 128), bar);
       if (l == 0)
-        bulk_in(st + kStageA, a.act[0] + (size_t)(r0 >> 3) * (IN / 8) * 128, image_bytes(rows, IN), bar);
+        bulk_in(st + kStageA, a.act[0] + (size_t)(tile0 + i) * image_bytes(R, IN) + off * group_bytes(IN), image_bytes(rows, IN), bar);
       else
-        for (int g = 0; g < groups; ++g)
-          bulk_in(st + kStageA + (uint32_t)g * 2048u, a.act[l] + ((size_t)(r0 >> 3) + g) * (W / 8) * 128 + (size_t)side * 2048, 2048u,
-                  bar);
+        bulk_in(st + kStageA, a.act[l] + (size_t)(tile0 + i) * image_bytes(R, W) + (size_t)side * image_bytes(R, 128) + off * group_bytes(W),
+                image_bytes(rows, 128), bar);
     };
     for (; issued < nsub && issued < BSTAGES; ++issued) copy(issued);
     for (; used < nsub; ++used) {
-      const int sl = used % BSTAGES, rows = min(KSUB, rend - rbeg - used * KSUB);
+      const int sl = used % BSTAGES, rows = rows_of(used);
       if (!mbar_wait(fullb + 8 * sl, (uint32_t)(used / BSTAGES) & 1u, &s_fail)) { s_fail = 12; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t st = base + (uint32_t)sl * kStage, kb = l == 0 ? (uint32_t)(IN / 8) * 128u : 2048u;
+      const uint32_t st = base + (uint32_t)sl * kStage, kb = group_bytes(N);
       const uint64_t da = make_desc(st, 2048u, 128u), db = make_desc(st + kStageA, kb, 128u);
       const uint64_t d1 = make_desc(base + SB_ONE, 128u, (uint32_t)(KSUB / 8) * 128u);
       for (int k = 0; k < rows; k += 16) {
