@@ -192,7 +192,7 @@ cudaError_t enqueue(cem_batch_ctx* h, cudaStream_t st, bool screened = false) {
   if (e != cudaSuccess) return e;
   e = mark(h, 2, st);
   if (e != cudaSuccess) return e;
-  e = launch_refit_batch(h->args_d, h->P, h->maxN, h->maxK, h->maxD, st);
+  e = launch_refit_batch(h->args_d, h->P, h->maxK, h->maxD, st);
   if (e != cudaSuccess) return e;
   return mark(h, 3, st);
 }

@@ -152,7 +152,7 @@ cudaError_t launch_refit(const RefitArgs& a, cudaStream_t st);
 // opts the refit kernel into its dynamic shared memory (once per device, before any capture)
 cudaError_t configure_refit();
 size_t refit_smem_bytes(int K, int D);
-cudaError_t launch_refit_batch(const RefitArgs* args_d, int n_problems, int maxN, int maxK, int maxD, cudaStream_t st);
+cudaError_t launch_refit_batch(const RefitArgs* args_d, int n_problems, int maxK, int maxD, cudaStream_t st);
 // batched sampling: problem p draws N_p rows from means[p*18..], chols[p*324..]
 // (D_p x D_p row-major) at Philox iteration tracks[p].iter
 cudaError_t launch_sample_batch(const BatchProblem* probs_d, int n_problems, int maxN, const float* means,

@@ -1,6 +1,5 @@
 // Exact selection of the smallest keys of a long array by one thread-block
-// cluster (1 to 8 CTAs of 1024 threads), shared by the top-k of the screening
-// pool and the elite selection.
+// cluster (1 to 8 CTAs of 1024 threads): the top-k of the screening pool.
 //
 // At most three histogram passes over 32-bit keys, 2048 bins each, that narrow
 // the range [lo, hi] of the wanted rank: the first over the span between the

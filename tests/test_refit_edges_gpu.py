@@ -1,6 +1,6 @@
-"""Elite selection and refit at the edges of the cluster's shares (counting up
-to 512 samples, one CTA up to 4096, four up to 16,384, eight beyond, 65,536
-keys in registers, 512 elites staged), against the oracle: indices exact,
+"""Elite selection and refit at the edges of its sizes (4096 keys in registers,
+512 elites staged, powers of two of the sort), with ties and costs that are not
+finite, against the oracle: indices exact,
 statistics within the roundings of their FP32 results (2^-24 relative, the
 covariance and its factor relative to their largest entry, with the factor's
 condition number allowed for)."""
