@@ -1,5 +1,5 @@
-"""Elite selection and refit at the edges of its sizes (4096 keys in registers,
-512 elites staged, powers of two of the sort), with ties and costs that are not
+"""Elite selection and refit at the edges of its sizes (16,384 keys in registers,
+512 elites staged, 1024 sorted in registers), with ties and costs that are not
 finite, against the oracle: indices exact,
 statistics within the roundings of their FP32 results (2^-24 relative, the
 covariance and its factor relative to their largest entry, with the factor's
