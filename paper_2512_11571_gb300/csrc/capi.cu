@@ -420,7 +420,7 @@ DevScene prepare(const cem_scene_desc& s, const cem_skeleton_desc& k) {
 
 int default_block(const cem_ctx* h, int N) {
   if (h->block > 0) return h->block;
-  return cem::default_rollout_block(N, h->host.kind, h->tpr);
+  return cem::default_rollout_block(N, h->host.kind, h->tpr, h->dr_on ? h->dr.M : 1);
 }
 
 // byte offsets of the solve state block (iters: history capacity)
@@ -677,23 +677,27 @@ int handle_read_result(cem_handle h, const cem_solve_params* p, SolveBuffers* b,
 int validate_descriptors(const cem_scene_desc* s, const cem_skeleton_desc* k) { return validate(s, k); }
 DevScene prepare_scene(const cem_scene_desc& s, const cem_skeleton_desc& k) { return prepare(s, k); }
 int set_last_error(int code, const std::string& msg) { return fail(code, msg); }
-int default_rollout_block(int N, int kind, int tpr) {
+int default_rollout_block(int N, int kind, int tpr, int envs) {
   // spread small batches over every SM scheduler: CTAs of 16 threads (each
-  // half-warp its own warp, 4 schedulers per SM) until the schedulers all
-  // have work, larger CTAs after that, up to 128 threads (measured on the
-  // push workload: 0.505 ms with 16 threads per CTA at N = 4096, 0.526 ms
-  // with 32 or 64; at N = 196,608 128 threads are 4 % faster than 256)
+  // half-warp its own warp, 4 schedulers per SM) up to one and a half warps a
+  // scheduler, larger CTAs after that, up to 128 threads.  Push, us with 16 /
+  // 32 / 64 threads: N = 4096 565 / 587 / 585, N = 8192 570 / 596 / 584, N =
+  // 16384 625 / 599 / 586; at N = 196,608 128 threads are 4 % faster than 256.
+  // The environments of a randomised sample are rollouts of their own here:
+  // 1000 push samples in 8 environments 577 / 614 / 627, 1500 576 / 617 / 619.
   int sms = 152;
   int dev = 0;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const long long R = (long long)N * envs;
   int b = 16;
-  while (b < 128 && (N + 2 * b - 1) / (2 * b) >= 4 * sms) b *= 2;
+  while (b < 128 && (R + b - 1) / b > 6 * sms) b *= 2;
   if (kind == CEM_SCENE_PICKPLACE && tpr == 1) {
     // pick-and-place lanes spend long stretches in different actions, so a
     // warp pays for its lanes' different branches one after another: fewer
     // lanes per warp, about 14 warps per SM (3.5 per scheduler), measured
-    // 6.7 ms against 7.5 ms at N = 4096 (2 lanes) and equal at N = 16384
-    const double target = (double)N / (14.0 * sms);
+    // 6.7 ms against 7.5 ms at N = 4096 (2 lanes) and equal at N = 16384; 3.0
+    // against 3.9 ms for 256 samples in 8 environments (8 lanes, one sample's)
+    const double target = (double)R / (14.0 * sms);
     int s = 2;
     while (s < 256 && s * 1.41 < target) s *= 2;
     if (s < b) b = s;

@@ -1353,11 +1353,19 @@ __device__ __noinline__ void quadratic_cost(const DevScene& s, const float* __re
   cls_out = isfinite(J) ? 0 : 3;
 }
 
+// The scene into shared memory, 16 bytes a load; a planar scene's head alone
+// (everything before the static geometry, which it does not have).  The CTAs
+// are small: word by word and whole, it took 16 threads 8 of the 73 us of 400
+// reach steps.
+template <int KIND>
 __device__ __forceinline__ void stage_scene(const DevScene* __restrict__ g, DevScene& sh) {
-  const int words = (int)(sizeof(DevScene) / 4);
-  const uint32_t* src = reinterpret_cast<const uint32_t*>(g);
-  uint32_t* dst = reinterpret_cast<uint32_t*>(&sh);
-  for (int i = threadIdx.x; i < words; i += blockDim.x) dst[i] = src[i];
+  constexpr bool kHead = KIND == CEM_SCENE_REACH || KIND == CEM_SCENE_PUSH;
+  constexpr int n = (int)((kHead ? offsetof(DevScene, geom_nslab) + 15 : sizeof(DevScene)) / 16);
+  static_assert(sizeof(DevScene) % 16 == 0 && alignof(DevScene) == 16, "copied by 16 bytes");
+  const uint4* src = reinterpret_cast<const uint4*>(g);
+  uint4* dst = reinterpret_cast<uint4*>(&sh);
+#pragma unroll 4
+  for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = src[i];
   __syncthreads();
 }
 
@@ -1379,7 +1387,7 @@ __global__ void __launch_bounds__(256, rollout_min_ctas<KIND>()) rollout_kernel(
                                                       float* __restrict__ J, uint8_t* __restrict__ cls,
                                                       float* __restrict__ trace) {
   __shared__ DevScene s;
-  stage_scene(scene_g, s);
+  stage_scene<KIND>(scene_g, s);
   const int n = (int)((blockIdx.x * blockDim.x + threadIdx.x) / G);
   if (n >= N) return;
   const float* row = theta + (size_t)n * s.D;
@@ -1410,7 +1418,7 @@ __global__ void __launch_bounds__(256, rollout_min_ctas<KIND>()) rollout_dr_kern
                                                          float* __restrict__ J, uint8_t* __restrict__ cls,
                                                          const DrArgs dr) {
   __shared__ DevScene s;
-  stage_scene(scene_g, s);
+  stage_scene<KIND>(scene_g, s);
   const int M = dr.M;
   const int t = (int)(blockIdx.x * blockDim.x + threadIdx.x);
   const int n = t / M, m = t & (M - 1);
@@ -1881,7 +1889,7 @@ cudaError_t launch_rollout(const DevScene* s_d, int kind, const float* theta, in
     return dispatch<false>(s_d, kind, theta, N, 0, J, cls, nullptr, block, tpr, st, astar);
   if (N <= 0) return cudaSuccess;
   if (dr->M < 1 || dr->M > 32 || (dr->M & (dr->M - 1))) return cudaErrorInvalidValue;
-  const int bt = block < 32 ? 32 : block;  // whole warps, so environment groups stay aligned
+  const int bt = block < dr->M ? dr->M : block;  // (both powers of two below 32: whole environment groups)
   const long long threads = (long long)N * dr->M;
   const int grid = (int)((threads + bt - 1) / bt);
   switch (kind) {
