@@ -47,10 +47,9 @@ struct B2 {
 };
 
 // Implicit Coulomb clamp of the trial velocity (branch-free): stick if the
-// speed is within mu g dt, else remove mu g dt along the velocity; the same
+// speed (squared: v2) is within mu g dt, else remove mu g dt along the velocity; the same
 // for the spin with capacity mu m g rbar dt / I.
-__device__ __forceinline__ void ground_clamp(B2& b, float cap, float cap2, float wcap) {
-  const float v2 = b.vx * b.vx + b.vy * b.vy;
+__device__ __forceinline__ void ground_clamp(B2& b, float v2, float cap, float cap2, float wcap) {
   const float f = v2 > cap2 ? 1.0f - cap * rsqrtf(v2) : 0.0f;
   b.vx *= f;
   b.vy *= f;
@@ -186,6 +185,15 @@ __device__ __forceinline__ void put_trace(float* tr, int step, const float* v, i
   for (int i = 0; i < TW; ++i) o[i] = i < nv ? v[i] : 0.0f;
 }
 
+// kp e - kd v.  The step's arithmetic is written out with its roundings (which
+// products are fused), so that every instantiation and any arrangement of the
+// code around it simulates the same trajectory bit for bit.
+__device__ __forceinline__ float pd_law(float kp, float e, float kd, float v) {
+  return __fmaf_rn(kp, e, -__fmul_rn(kd, v));
+}
+// x^2 + y^2
+__device__ __forceinline__ float sq2(float x, float y) { return __fmaf_rn(x, x, __fmul_rn(y, y)); }
+
 // ------------------------------------------------------------- reach / push
 // The success test compares squared distances; the square roots are taken
 // only at the step that succeeds (for the interpolated crossing time).
@@ -194,9 +202,67 @@ __device__ __forceinline__ void put_trace(float* tr, int step, const float* v, i
 // the same instructions and return bit-identical results.
 // smu / sm: friction and manipulated-body mass scales of a randomised
 // environment (exactly 1 otherwise, which leaves every value unchanged).
-template <bool HAS_BLOCK, bool TRACE>
-__device__ __noinline__ void planar_rollout(const DevScene& s, const float* __restrict__ row, int T, float smu, float sm,
-                                            float& J_out, int& cls_out, float* tr) {
+// A moveTo without a block.  Bound by the latency of one step's chain (one warp
+// a scheduler at most): an action is loaded where its predecessor ends, so that
+// a step has a single branch, and a search of 256 samples, ten iterations, takes
+// 583 us; with the load asked for at the start of each step and the end of the
+// action in a branch of its own, 649.
+template <bool TRACE>
+__device__ __noinline__ void reach_rollout(const DevScene& s, const float* __restrict__ row, int T, float smu,
+                                           float& J_out, int& cls_out, float* tr) {
+  const float dt = s.dt, eps2 = s.eps * s.eps;
+  const float mb = s.mb, Ib = s.Ib, dt_mb = s.dt_mb, dt_Ib = s.dt_Ib;
+  const float bcap = s.base_cap * smu, bcap2 = bcap * bcap, bwcap = s.base_wcap * smu;
+  const float ykp = s.yaw_kp, ykd = s.yaw_kd;
+  B2 b{s.base_start[0], s.base_start[1], s.base_start[2], s.base_v0[0], s.base_v0[1], s.base_v0[2]};
+  const int L = s.n_act;
+  int a = 0;
+  float gx = 0.f, gy = 0.f, kp = 0.f, kd = 0.f, rx = 0.f, ry = 0.f, yaw_t = 0.f;
+  float t_done = (float)T * dt, d2_cur = 0.0f;
+  auto load_action = [&](int ai) {
+    const int o = s.act_off[ai];
+    gx = s.act_nom[ai][0] + theta_at(s, row, o);
+    gy = s.act_nom[ai][1] + theta_at(s, row, o + 1);
+    kp = theta_at(s, row, o + 2);
+    kd = 2.0f * sqrtf(kp);
+    rx = s.act_ref[ai] ? gx : s.act_nom[ai][0];
+    ry = s.act_ref[ai] ? gy : s.act_nom[ai][1];
+    yaw_t = s.act_yaw[ai];
+    d2_cur = sq2(b.x - rx, b.y - ry);
+  };
+  load_action(0);
+  for (int step = 0; step < T; ++step) {
+    b.vx += dt_mb * (mb * pd_law(kp, gx - b.x, kd, b.vx));
+    b.vy += dt_mb * (mb * pd_law(kp, gy - b.y, kd, b.vy));
+    b.w += dt_Ib * (Ib * pd_law(ykp, yaw_t - b.psi, ykd, b.w));
+    ground_clamp(b, sq2(b.vx, b.vy), bcap, bcap2, bwcap);
+    b.x += b.vx * dt;
+    b.y += b.vy * dt;
+    b.psi += b.w * dt;
+    const float d2_old = d2_cur;
+    d2_cur = sq2(b.x - rx, b.y - ry);
+    if (a < L && d2_cur <= eps2) {
+      if (a == L - 1) t_done = success_time(s, step, sqrtf(d2_old), sqrtf(d2_cur));
+      ++a;
+      if (a < L) load_action(a);
+    }
+    if (TRACE) {
+      const float v[13] = {b.x, b.y, b.psi, b.vx, b.vy, b.w, s.block_start[0], s.block_start[1],
+                           s.block_start[2], s.block_v0[0], s.block_v0[1], s.block_v0[2], (float)a};
+      put_trace(tr, step, v, 13);
+    }
+  }
+  const float ex = b.x - s.goal_center[0], ey = b.y - s.goal_center[1];
+  const float dist = sqrtf(ex * ex + ey * ey);
+  const float J = s.w_time * t_done + s.w_goal * dist;
+  J_out = J;
+  cls_out = a == L ? (dist <= s.eps ? 0 : 1) : 2;
+  if (!isfinite(J)) cls_out = 3;
+}
+
+template <bool TRACE>
+__device__ __noinline__ void push_rollout(const DevScene& s, const float* __restrict__ row, int T, float smu, float sm,
+                                          float& J_out, int& cls_out, float* tr) {
   // loop invariants in registers
   const float dt = s.dt, eps2 = s.eps * s.eps;
   const float mb = s.mb, Ib = s.Ib, dt_mb = s.dt_mb, dt_Ib = s.dt_Ib;
@@ -208,7 +274,7 @@ __device__ __noinline__ void planar_rollout(const DevScene& s, const float* __re
   const float kwcap = s.block_wcap * smu;
   const float kc = s.k_contact, cc = s.c_contact, mu_dt = s.contact_mu * smu * s.dt, flim = s.force_limit;
   const float inv_mb = 1.0f / s.mb, inv_Ib = 1.0f / s.Ib;
-  const float inv_mk = HAS_BLOCK ? 1.0f / (s.mk * sm) : 0.0f, inv_Ik = HAS_BLOCK ? 1.0f / (s.Ik * sm) : 0.0f;
+  const float inv_mk = 1.0f / (s.mk * sm), inv_Ik = 1.0f / (s.Ik * sm);
   // broad phase: the block's bounding circle (radius rk) against the base
   // rectangle, in the base frame; the hardware sine/cosine is off by < 1e-6,
   // so a 1e-4 m margin keeps the test conservative (it never rejects a pair
@@ -241,70 +307,64 @@ __device__ __noinline__ void planar_rollout(const DevScene& s, const float* __re
     float fkx = 0.f, fky = 0.f, tk = 0.f, Fn = 0.f;
     float rax = 0.f, ray = 0.f, rbx = 0.f, rby = 0.f, nx = 0.f, ny = 0.f;
     bool hit = false;
-    if (HAS_BLOCK) {
-      const float cdx = k.x - b.x, cdy = k.y - b.y;
-      float sbp, cbp;
-      yaw_sincos(b.psi, &sbp, &cbp);
-      if (fabsf(cdx * cbp + cdy * sbp) < reach_u && fabsf(cdy * cbp - cdx * sbp) < reach_w) {
-        float dep, qx, qy;
-        hit = sat_rect(b, sbp, cbp, bhx, bhy, k, khx, khy, nx, ny, dep, qx, qy);
-        if (hit) {
-          rax = qx - b.x;
-          ray = qy - b.y;
-          rbx = qx - k.x;
-          rby = qy - k.y;
-          const float vrx = (k.vx - k.w * rby) - (b.vx - b.w * ray);
-          const float vry = (k.vy + k.w * rbx) - (b.vy + b.w * rax);
-          const float vn = vrx * nx + vry * ny;
-          Fn = fmaxf(0.0f, kc * dep - cc * vn);
-          fkx = Fn * nx;
-          fky = Fn * ny;
-          fx -= fkx;
-          fy -= fky;
-          tq -= cross2(rax, ray, fkx, fky);
-          tk = cross2(rbx, rby, fkx, fky);
-          const float over = Fn - flim;
-          if (over > 0.0f) viol += over * dt;
-        }
+    const float cdx = k.x - b.x, cdy = k.y - b.y;
+    float sbp, cbp;
+    yaw_sincos(b.psi, &sbp, &cbp);
+    if (fabsf(cdx * cbp + cdy * sbp) < reach_u && fabsf(cdy * cbp - cdx * sbp) < reach_w) {
+      float dep, qx, qy;
+      hit = sat_rect(b, sbp, cbp, bhx, bhy, k, khx, khy, nx, ny, dep, qx, qy);
+      if (hit) {
+        rax = qx - b.x;
+        ray = qy - b.y;
+        rbx = qx - k.x;
+        rby = qy - k.y;
+        const float vrx = (k.vx - k.w * rby) - (b.vx - b.w * ray);
+        const float vry = (k.vy + k.w * rbx) - (b.vy + b.w * rax);
+        const float vn = vrx * nx + vry * ny;
+        Fn = fmaxf(0.0f, kc * dep - cc * vn);
+        fkx = Fn * nx;
+        fky = Fn * ny;
+        fx -= fkx;
+        fy -= fky;
+        tq -= cross2(rax, ray, fkx, fky);
+        tk = cross2(rbx, rby, fkx, fky);
+        const float over = Fn - flim;
+        if (over > 0.0f) viol += over * dt;
       }
     }
     b.vx += dt_mb * fx;
     b.vy += dt_mb * fy;
     b.w += dt_Ib * tq;
-    if (HAS_BLOCK) {
-      k.vx += dt_mk * fkx;
-      k.vy += dt_mk * fky;
-      k.w += dt_Ik * tk;
-      if (hit && Fn > 0.0f) {
-        const float tx = -ny, ty = nx;
-        const float vrx = (k.vx - k.w * rby) - (b.vx - b.w * ray);
-        const float vry = (k.vy + k.w * rbx) - (b.vy + b.w * rax);
-        const float vt = vrx * tx + vry * ty;
-        const float ca = cross2(rax, ray, tx, ty), cb = cross2(rbx, rby, tx, ty);
-        const float inv_m = inv_mb + inv_mk + ca * ca * inv_Ib + cb * cb * inv_Ik;
-        // fast division (2 ulp; inv_m is an inverse mass sum of order 1..10):
-        // this chain sets the step latency of every warp with a block contact
-        const float jm = fminf(mu_dt * Fn, __fdividef(fabsf(vt), inv_m));
-        const float jt = vt > 0.0f ? -jm : jm;
-        const float jx = jt * tx, jy = jt * ty;
-        k.vx += jx * inv_mk;
-        k.vy += jy * inv_mk;
-        k.w += cross2(rbx, rby, jx, jy) * inv_Ik;
-        b.vx -= jx * inv_mb;
-        b.vy -= jy * inv_mb;
-        b.w -= cross2(rax, ray, jx, jy) * inv_Ib;
-      }
-      ground_clamp(k, kcap, kcap2, kwcap);
+    k.vx += dt_mk * fkx;
+    k.vy += dt_mk * fky;
+    k.w += dt_Ik * tk;
+    if (hit && Fn > 0.0f) {
+      const float tx = -ny, ty = nx;
+      const float vrx = (k.vx - k.w * rby) - (b.vx - b.w * ray);
+      const float vry = (k.vy + k.w * rbx) - (b.vy + b.w * rax);
+      const float vt = vrx * tx + vry * ty;
+      const float ca = cross2(rax, ray, tx, ty), cb = cross2(rbx, rby, tx, ty);
+      const float inv_m = inv_mb + inv_mk + ca * ca * inv_Ib + cb * cb * inv_Ik;
+      // fast division (2 ulp; inv_m is an inverse mass sum of order 1..10):
+      // this chain sets the step latency of every warp with a block contact
+      const float jm = fminf(mu_dt * Fn, __fdividef(fabsf(vt), inv_m));
+      const float jt = vt > 0.0f ? -jm : jm;
+      const float jx = jt * tx, jy = jt * ty;
+      k.vx += jx * inv_mk;
+      k.vy += jy * inv_mk;
+      k.w += cross2(rbx, rby, jx, jy) * inv_Ik;
+      b.vx -= jx * inv_mb;
+      b.vy -= jy * inv_mb;
+      b.w -= cross2(rax, ray, jx, jy) * inv_Ib;
     }
-    ground_clamp(b, bcap, bcap2, bwcap);
+    ground_clamp(k, k.vx * k.vx + k.vy * k.vy, kcap, kcap2, kwcap);
+    ground_clamp(b, b.vx * b.vx + b.vy * b.vy, bcap, bcap2, bwcap);
     b.x += b.vx * dt;
     b.y += b.vy * dt;
     b.psi += b.w * dt;
-    if (HAS_BLOCK) {
-      k.x += k.vx * dt;
-      k.y += k.vy * dt;
-      k.psi += k.w * dt;
-    }
+    k.x += k.vx * dt;
+    k.y += k.vy * dt;
+    k.psi += k.w * dt;
     if (a < L) {
       const float d2_new = (b.x - rx) * (b.x - rx) + (b.y - ry) * (b.y - ry);
       if (d2_new <= eps2) {
@@ -320,20 +380,11 @@ __device__ __noinline__ void planar_rollout(const DevScene& s, const float* __re
     }
   }
   const bool complete = a == L;
-  bool goal;
-  float J;
-  if (!HAS_BLOCK) {
-    const float ex = b.x - s.goal_center[0], ey = b.y - s.goal_center[1];
-    const float dist = sqrtf(ex * ex + ey * ey);
-    goal = dist <= s.eps;
-    J = s.w_time * t_done + s.w_goal * dist;
-  } else {
-    const float ax = fabsf(k.x - s.goal_center[0]), ay = fabsf(k.y - s.goal_center[1]);
-    const float ex = fmaxf(ax - s.goal_half[0], 0.0f), ey = fmaxf(ay - s.goal_half[1], 0.0f);
-    const float dist = sqrtf(ex * ex + ey * ey);
-    goal = ax <= s.goal_half[0] && ay <= s.goal_half[1];
-    J = s.w_time * t_done + s.w_goal * dist + s.w_viol * viol;
-  }
+  const float ax = fabsf(k.x - s.goal_center[0]), ay = fabsf(k.y - s.goal_center[1]);
+  const float ex = fmaxf(ax - s.goal_half[0], 0.0f), ey = fmaxf(ay - s.goal_half[1], 0.0f);
+  const float dist = sqrtf(ex * ex + ey * ey);
+  const bool goal = ax <= s.goal_half[0] && ay <= s.goal_half[1];
+  const float J = s.w_time * t_done + s.w_goal * dist + s.w_viol * viol;
   J_out = J;
   cls_out = complete ? (goal ? 0 : 1) : 2;
   if (!isfinite(J)) cls_out = 3;
@@ -1001,12 +1052,6 @@ __device__ __forceinline__ void arm_ee_velocity(const DevScene& s, float q1, flo
   vy = bvy + dr * sb;
 }
 
-// kp e - kd v.  The step's arithmetic is written out with its roundings (which
-// products are fused), so that every instantiation and any arrangement of the
-// code around it simulates the same trajectory bit for bit.
-__device__ __forceinline__ float pd_law(float kp, float e, float kd, float v) {
-  return __fmaf_rn(kp, e, -__fmul_rn(kd, v));
-}
 __device__ __forceinline__ float norm2(float x, float y, float z) {
   return __fmaf_rn(z, z, __fmaf_rn(x, x, __fmul_rn(y, y)));
 }
@@ -1395,8 +1440,8 @@ __global__ void __launch_bounds__(256, rollout_min_ctas<KIND>()) rollout_kernel(
   const int T = TRACE ? steps : s.T;
   float Jn;
   int c;
-  if (KIND == CEM_SCENE_REACH) planar_rollout<false, TRACE>(s, row, T, 1.0f, 1.0f, Jn, c, tr);
-  else if (KIND == CEM_SCENE_PUSH) planar_rollout<true, TRACE>(s, row, T, 1.0f, 1.0f, Jn, c, tr);
+  if (KIND == CEM_SCENE_REACH) reach_rollout<TRACE>(s, row, T, 1.0f, Jn, c, tr);
+  else if (KIND == CEM_SCENE_PUSH) push_rollout<TRACE>(s, row, T, 1.0f, 1.0f, Jn, c, tr);
   else if (KIND == CEM_SCENE_PICKPLACE) {
     if (AS) pickplace_any<G, TRACE>(s, row, T, 1.0f, 1.0f, Jn, c, tr);
     else pickplace_rollout<G, TRACE, false>(s, row, T, 1.0f, 1.0f, Jn, c, tr);  // the scene has the PD base
@@ -1431,8 +1476,8 @@ __global__ void __launch_bounds__(256, rollout_min_ctas<KIND>()) rollout_dr_kern
   const float* row = theta + (size_t)n * s.D;
   float Jn;
   int c;
-  if (KIND == CEM_SCENE_REACH) planar_rollout<false, false>(s, row, s.T, smu, sm, Jn, c, nullptr);
-  else if (KIND == CEM_SCENE_PUSH) planar_rollout<true, false>(s, row, s.T, smu, sm, Jn, c, nullptr);
+  if (KIND == CEM_SCENE_REACH) reach_rollout<false>(s, row, s.T, smu, Jn, c, nullptr);
+  else if (KIND == CEM_SCENE_PUSH) push_rollout<false>(s, row, s.T, smu, sm, Jn, c, nullptr);
   else pickplace_any<1, false>(s, row, s.T, smu, sm, Jn, c, nullptr);
   const int lane = threadIdx.x & 31;
   const unsigned gmask = M == 32 ? 0xffffffffu : (((1u << M) - 1u) << (lane & ~(M - 1)));
@@ -1645,8 +1690,8 @@ __global__ void __launch_bounds__(256, 2) rollout_persistent_kernel(const DevSce
           float Jn;
           int c;
           switch (s.kind) {
-            case CEM_SCENE_REACH: planar_rollout<false, false>(s, row, s.T, smu, sm, Jn, c, nullptr); break;
-            case CEM_SCENE_PUSH: planar_rollout<true, false>(s, row, s.T, smu, sm, Jn, c, nullptr); break;
+            case CEM_SCENE_REACH: reach_rollout<false>(s, row, s.T, smu, Jn, c, nullptr); break;
+            case CEM_SCENE_PUSH: push_rollout<false>(s, row, s.T, smu, sm, Jn, c, nullptr); break;
             default: pickplace_batch<1, AS>(s, row, smu, sm, Jn, c); break;
           }
           for (int o = 1; o < M; o <<= 1) {
@@ -1686,8 +1731,8 @@ __global__ void __launch_bounds__(256, 2) rollout_persistent_kernel(const DevSce
         float Jn;
         int c;
         switch (s.kind) {
-          case CEM_SCENE_REACH: planar_rollout<false, false>(s, row, s.T, 1.0f, 1.0f, Jn, c, nullptr); break;
-          case CEM_SCENE_PUSH: planar_rollout<true, false>(s, row, s.T, 1.0f, 1.0f, Jn, c, nullptr); break;
+          case CEM_SCENE_REACH: reach_rollout<false>(s, row, s.T, 1.0f, Jn, c, nullptr); break;
+          case CEM_SCENE_PUSH: push_rollout<false>(s, row, s.T, 1.0f, 1.0f, Jn, c, nullptr); break;
           case CEM_SCENE_PICKPLACE: pickplace_batch<1, AS>(s, row, 1.0f, 1.0f, Jn, c); break;
           default: quadratic_cost(s, row, Jn, c); break;
         }
