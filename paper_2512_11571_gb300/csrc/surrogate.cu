@@ -9,8 +9,10 @@
 // candidate pool, score it, and roll out only the best-scored candidates;
 // elites still come from simulated costs only.
 //
-// Dense layers run on the tensor cores through one tiled GEMM kernel
-// (128 x 128 x 32 tiles, 8 warps, mma m16n8k16 BF16 -> FP32) with fused
+// Networks of 48-256x4 train through the fused step of mlp_train.cu (three
+// launches a step) and score through mlp_tc.cu; other shapes, and the paths a
+// caller selects, run layer by layer on gemm_tc.cu or on the tiled GEMM kernel
+// here (128 x 128 x 32 tiles, 8 warps, mma m16n8k16 BF16 -> FP32) with fused
 // epilogues: bias + GELU (forward, also keeping the FP32 pre-activation for
 // the backward pass) and GELU' (backward).  Every reduction (loss, bias and
 // output-layer gradients, target statistics) runs in a fixed order, so
