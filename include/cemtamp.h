@@ -453,8 +453,11 @@ int cem_surrogate_set_forward_path(cem_surrogate_handle s, int path);
 /* Failure-detection test hook: while on != 0, tcgen05 forwards leave their
  * first weight-copy barrier without its arrival, so every CTA's first
  * pipeline wait runs out after 1 s with nothing in flight; the CTA then
- * frees its TMEM, writes NaN scores and sets status 1.  The context stays
- * usable; switch it off (0) for normal forwards. */
+ * frees its TMEM, writes NaN scores and sets status 1.  The fused training
+ * step does the same in its first launch (status 2), or, with on = 2, in its
+ * second (status 12); cem_surrogate_gradient and cem_surrogate_train then
+ * return CEM_ERR_TIMEOUT.  The context stays usable; switch it off (0) for
+ * normal calls. */
 int cem_surrogate_test_expire_wait(cem_surrogate_handle s, int on);
 /* The path inference takes now: 1 tiled GEMM, 2 tcgen05; -1 for NULL. */
 int cem_surrogate_forward_path(cem_surrogate_handle s);
@@ -487,19 +490,25 @@ int cem_surrogate_adamw_step(cem_surrogate_handle s, const float* grad_h, float 
  * state; get it to checkpoint.  get synchronises. */
 int cem_surrogate_set_adam_state(cem_surrogate_handle s, const float* m1_h, const float* m2_h, long long steps_taken);
 int cem_surrogate_get_adam_state(cem_surrogate_handle s, float* m1_h, float* m2_h, long long* steps_taken);
-/* Synchronises, writes and clears the tcgen05 forward's status word: 0, or
- * 1 / 2 if a wait for the weight copy / the MMAs expired.  A non-zero code
- * also makes cem_solve_screened return CEM_ERR_TIMEOUT. */
+/* Synchronises, writes and clears the status word of the tcgen05 kernels: 0,
+ * or the code of an expired wait: forward 1 / 2 (the weight copy / the MMAs),
+ * which also makes cem_solve_screened return CEM_ERR_TIMEOUT; fused training
+ * step 1 to 9 (its first launch: rows) and 11 to 13 (its second: weights). */
 int cem_surrogate_status(cem_surrogate_handle s, int* status_h);
 /* Full-batch gradient of mean((out - (t - mu)/sigma)^2) over M rows into
- * grad_h (num_params floats) and the loss into *loss_h.  Synchronous. */
+ * grad_h (num_params floats) and the loss into *loss_h.  Synchronous.
+ * CEM_ERR_TIMEOUT if a wait of the fused training step expired (48-256x4 on
+ * gemm path 0 or 2; cem_surrogate_status has the code); nothing is written. */
 int cem_surrogate_gradient(cem_surrogate_handle s, const float* x_d, const float* t_d, int M, float* grad_h,
                            float* loss_h);
 /* `steps` AdamW steps (beta 0.9/0.999, eps 1e-8, decoupled decay on
  * weights) on minibatches of `batch` rows drawn with replacement by Philox
  * from (x_d[M][48], t_d[M]); normalize != 0 first sets (mu, sigma) to the
  * targets' mean and standard deviation.  loss_hist_h (steps floats) may be
- * NULL.  Synchronous. */
+ * NULL.  Synchronous.  CEM_ERR_TIMEOUT if a wait of the fused training step
+ * expired (as in cem_surrogate_gradient): that step and all after it change
+ * nothing, so the parameters and the optimiser's state are those of the steps
+ * before it; no losses are written. */
 int cem_surrogate_train(cem_surrogate_handle s, const float* x_d, const float* t_d, int M, int batch, int steps,
                         float lr, float weight_decay, uint64_t seed, int normalize, float* loss_hist_h);
 /* Training target of simulated samples: t_d[n] = log(1 + max(J_d[n], 0) +

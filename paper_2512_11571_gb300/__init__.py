@@ -821,7 +821,7 @@ def cem_surrogate_set_forward_path(s, path):
 
 
 def cem_surrogate_test_expire_wait(s, on):
-    _check(load().cem_surrogate_test_expire_wait(s, int(bool(on))))
+    _check(load().cem_surrogate_test_expire_wait(s, on if isinstance(on, int) else int(bool(on))))
 
 
 def cem_surrogate_forward_path(s):
@@ -967,7 +967,8 @@ class Surrogate:
         return cem_surrogate_gemm_path(self.h)
 
     def test_expire_wait(self, on):
-        """Failure-detection hook: make the tcgen05 forward's first wait run out."""
+        """Failure-detection hook: make a wait of the tcgen05 forward and of the
+        fused training step run out (which one: see cemtamp.h)."""
         cem_surrogate_test_expire_wait(self.h, on)
 
     def adamw_step(self, grad, lr=1e-3, weight_decay=1e-4):

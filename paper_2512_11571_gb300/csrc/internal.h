@@ -308,6 +308,12 @@ __host__ __device__ constexpr int train_part4(int l) {
   return l == 0 ? 0 : (kTrainIn / 4 + (l - 1) * (kTrainWidth / 4)) * kTrainWidth;
 }
 constexpr int kTrainPart4 = train_part4(kTrainDepth);
+// what a call's steps report (cleared by train_pack)
+struct TrainOut {
+  float loss;  // sum of the last step's squared residuals
+  int status;  // 0, or the code of the first bounded wait that expired: that step and all later ones change nothing
+  int steps;   // optimiser steps applied
+};
 struct TrainArgs {
   // data: FP32 rows x[][48] and targets t[]; the step's rows are drawn from
   // draw_from of them (Philox on the step), or, if that is 0, the first
@@ -341,16 +347,16 @@ struct TrainArgs {
   float* g;
   float* m1;
   float* m2;
-  float* loss_d;  // sum of the squared residuals
-  float* hist;    // per step (may be null)
+  float* hist;  // squared residuals per step (may be null)
+  TrainOut* out;
   float lr, b1, b2, eps, wd;
   int* step_d;
   long long* adam_t_d;
-  int* status;
+  int expire_test;  // failure-detection test: whose copy to leave out, 1 rows, 2 weights
 };
 bool train_supported(int in_dim, int width, int depth);
 size_t train_pack_bytes();
-// the weight image from pb (before the first step of a call)
+// the weight image from pb and a cleared out (before the first step of a call)
 cudaError_t train_pack(const TrainArgs& a, cudaStream_t st);
 cudaError_t train_step(const TrainArgs& a, cudaStream_t st);
 

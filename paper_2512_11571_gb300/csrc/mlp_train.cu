@@ -38,8 +38,11 @@
 // of the same rows, bias, GELU and GELU' in FP32 afterwards, every sum in the
 // same fixed order), so both train the same network bit for bit.
 //
-// Waits are bounded (1 s of global time); on expiry the CTA sets *status,
+// Waits are bounded (1 s of global time); on expiry the CTA sets out->status,
 // waits (bounded) for its own copies and MMAs, frees its TMEM and returns.
+// From then on the launches of the call do nothing: rows and weights give up
+// at their first look at the status and update writes nothing, so the
+// parameters are those after the last whole step.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -173,6 +176,10 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
 // wrote or read only after grid_wait, which returns when that one is complete.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// The status is looked at while the first copies are under way (it costs no
+// time there) and set by the first that gives up.
+__device__ __forceinline__ int step_status(const TrainArgs& a) { return *(volatile int*)&a.out->status; }
+__device__ __forceinline__ void step_failed(const TrainArgs& a, int code) { atomicCAS(&a.out->status, 0, code); }
 __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&h);
@@ -251,7 +258,9 @@ __global__ void __launch_bounds__(THREADS, 1) train_rows_kernel(const TrainArgs 
         copying[h] = false;
         return true;
       };
-      load_half(0, weight_base(0), kW0Bytes);
+      // (the failure-detection test leaves the first weights' barrier without its arrival)
+      if (a.expire_test != 1) load_half(0, weight_base(0), kW0Bytes);
+      if (step_status(a)) fail = 10;
       for (int l = 0; l < DEPTH && !fail; ++l) {
         const int K = l == 0 ? IN : W;
         // layer l's input is written and its accumulators are drained
@@ -469,7 +478,7 @@ __global__ void __launch_bounds__(THREADS, 1) train_rows_kernel(const TrainArgs 
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (s_fail && tid == 0) atomicExch(a.status, s_fail);
+  if (s_fail && tid == 0) step_failed(a, s_fail);
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kColsA));
 }
 
@@ -576,8 +585,10 @@ __global__ void __launch_bounds__(BTHREADS, 2) train_weights_kernel(const TrainA
         bulk_in(st + kStageA, a.act[l] + (size_t)(tile0 + i) * image_bytes(R, W) + (size_t)side * image_bytes(R, 128) + off * group_bytes(W),
                 image_bytes(rows, 128), bar);
     };
-    for (; issued < nsub && issued < BSTAGES; ++issued) copy(issued);
-    for (; used < nsub; ++used) {
+    // (the failure-detection test leaves the first copies out)
+    for (; issued < nsub && issued < BSTAGES && a.expire_test != 2; ++issued) copy(issued);
+    if (step_status(a)) s_fail = 10;
+    for (; used < nsub && !s_fail; ++used) {
       const int sl = used % BSTAGES, rows = rows_of(used);
       if (!mbar_wait(fullb + 8 * sl, (uint32_t)(used / BSTAGES) & 1u, &s_fail)) { s_fail = 12; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -640,7 +651,7 @@ __global__ void __launch_bounds__(BTHREADS, 2) train_weights_kernel(const TrainA
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (s_fail && tid == 0) atomicExch(a.status, s_fail);
+  if (s_fail && tid == 0) step_failed(a, s_fail);
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kColsB));
 }
 
@@ -665,7 +676,9 @@ __global__ void __launch_bounds__(CTHREADS) train_update_kernel(const TrainArgs 
     s_c[0] = 1.0f - powf(a.b1, t);
     s_c[1] = 1.0f - powf(a.b2, t);
   }
+  const bool failed = step_status(a) != 0;  // (set by earlier launches only: the same in every thread)
   if (b >= kUpdate4) __syncthreads();
+  if (b >= kUpdate4 && failed) return;
   auto apply = [&](int i, float g, int decay) -> float {  // returns the new parameter
     if (!step) {
       a.g[i] = g;
@@ -695,6 +708,7 @@ __global__ void __launch_bounds__(CTHREADS) train_update_kernel(const TrainArgs 
       s.z += v.z;
       s.w += v.w;
     }
+    if (failed) return;
     if (!step) {
       *reinterpret_cast<float4*>(a.g + i) = s;
       return;
@@ -757,8 +771,11 @@ __global__ void __launch_bounds__(CTHREADS) train_update_kernel(const TrainArgs 
         const float x = apply(i, red[0], 0);
         if (step) a.pb[i] = __float2bfloat16_rn(x);
       } else {
-        *a.loss_d = red[0];
-        if (step && a.hist) a.hist[*a.step_d - 1] = red[0];
+        a.out->loss = red[0];
+        if (step) {
+          a.out->steps += 1;
+          if (a.hist) a.hist[*a.step_d - 1] = red[0];
+        }
       }
     }
   }
@@ -768,6 +785,7 @@ __global__ void __launch_bounds__(CTHREADS) train_update_kernel(const TrainArgs 
 // the update keeps it)
 __global__ void train_pack_kernel(const bf16* __restrict__ pb, const TrainArgs a) {
   const int l = blockIdx.y, K = l == 0 ? IN : W, i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (l == 0 && i == 0) *a.out = TrainOut{0.0f, 0, 0};
   if (i >= W * K) return;
   *reinterpret_cast<bf16*>(a.wpack_out + weight_base(l) + weight_off(i / K, i % K, K)) = pb[a.w_off[l] + i];
 }

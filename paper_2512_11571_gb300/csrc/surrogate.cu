@@ -963,7 +963,7 @@ int train_args(cem_surrogate_ctx* s, const float* x_d, const float* t_d, int bat
   const size_t gp = take(rows * W * 4 * kTrainDepth), dy = take(rows * 4), sq = take(rows * 4);
   const size_t part = take(sizeof(float) * 4 * (size_t)kTrainPart4 * a.chunks);
   const size_t bpart = take(sizeof(float) * W * kTrainDepth * a.chunks), cpart = take(sizeof(float) * W * a.tiles);
-  const size_t lpart = take(sizeof(float) * (((size_t)batch + 255) / 256)), loss = take(sizeof(float));
+  const size_t lpart = take(sizeof(float) * (((size_t)batch + 255) / 256)), out_at = take(sizeof(TrainOut));
   if (o > s->train_bytes || !s->train_work) {
     cudaFree(s->train_work);
     s->train_work = nullptr;
@@ -996,15 +996,21 @@ int train_args(cem_surrogate_ctx* s, const float* x_d, const float* t_d, int bat
   a.biaspart = reinterpret_cast<float*>(w + bpart);
   a.colpart = reinterpret_cast<float*>(w + cpart);
   a.losspart = reinterpret_cast<float*>(w + lpart);
-  a.loss_d = reinterpret_cast<float*>(w + loss);
+  a.out = reinterpret_cast<TrainOut*>(w + out_at);
   a.g = s->g;
   a.m1 = s->m1;
   a.m2 = s->m2;
   a.step_d = s->step_d;
   a.adam_t_d = s->adam_t_d;
-  a.status = s->tc_status;
+  a.expire_test = s->expire_test;
   *out = a;
   return CEM_OK;
+}
+
+// a fused call whose wait expired: the code for cem_surrogate_status, and the error
+int train_expired(cem_surrogate_ctx* s, int code) {
+  cudaMemcpy(s->tc_status, &code, sizeof(int), cudaMemcpyHostToDevice);
+  return fail(CEM_ERR_TIMEOUT, "surrogate training: a bounded wait on the tensor-core pipeline expired");
 }
 
 // scores of M rows, no activations kept: the fused tcgen05 kernel where the
@@ -1388,7 +1394,7 @@ int cem_surrogate_set_forward_path(cem_surrogate_handle s, int path) {
 
 int cem_surrogate_test_expire_wait(cem_surrogate_handle s, int on) {
   if (!s) return fail(CEM_ERR_INVALID_ARG, "null handle");
-  s->expire_test = on ? 1 : 0;
+  s->expire_test = on == 2 ? 2 : on ? 1 : 0;
   return CEM_OK;
 }
 
@@ -1451,17 +1457,19 @@ int cem_surrogate_gradient(cem_surrogate_handle s, const float* x_d, const float
   if (!s || !grad_h) return fail(CEM_ERR_INVALID_ARG, "null argument");
   if (M < 1 || M > (1 << 22)) return fail(CEM_ERR_UNSUPPORTED, "M must be in 1..2^22");
   if (!is_dev(x_d) || !is_dev(t_d)) return fail(CEM_ERR_INVALID_ARG, "x and t must be device pointers");
-  const float* loss_d = nullptr;  // (s->loss_d where it stays null)
+  TrainOut fused_out;
+  const bool fused = use_fused_train(s);
   if (s->gemm_path == 3) {
     int rc = gradient_f32(s, x_d, t_d, M);
     if (rc != CEM_OK) return rc;
-  } else if (use_fused_train(s)) {
+  } else if (fused) {
     TrainArgs a;
     int rc = train_args(s, x_d, t_d, M, &a);
     if (rc != CEM_OK) return rc;
     SUR_CUDA(train_pack(a, 0));
     SUR_CUDA(train_step(a, 0));
-    loss_d = a.loss_d;
+    SUR_CUDA(cudaMemcpy(&fused_out, a.out, sizeof(fused_out), cudaMemcpyDeviceToHost));
+    if (fused_out.status) return train_expired(s, fused_out.status);
   } else {
     int rc = load_features(s, x_d, M, 0);
     if (rc != CEM_OK) return rc;
@@ -1473,7 +1481,8 @@ int cem_surrogate_gradient(cem_surrogate_handle s, const float* x_d, const float
   SUR_CUDA(cudaMemcpy(grad_h, s->g, sizeof(float) * s->total, cudaMemcpyDeviceToHost));
   if (loss_h) {
     float l = 0.0f;
-    SUR_CUDA(cudaMemcpy(&l, loss_d ? loss_d : s->loss_d, sizeof(float), cudaMemcpyDeviceToHost));
+    if (fused) l = fused_out.loss;
+    else SUR_CUDA(cudaMemcpy(&l, s->loss_d, sizeof(float), cudaMemcpyDeviceToHost));
     *loss_h = l / M;
   }
   return CEM_OK;
@@ -1567,8 +1576,10 @@ int cem_surrogate_train(cem_surrogate_handle s, const float* x_d, const float* t
     if (exec) cudaGraphExecDestroy(exec);
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e == cudaSuccess) s->adam_step += steps;
-  if (hist_d && e == cudaSuccess) {
+  TrainOut fused_out{0.0f, 0, steps};
+  if (fused && steps > 0 && e == cudaSuccess) e = cudaMemcpy(&fused_out, ta.out, sizeof(fused_out), cudaMemcpyDeviceToHost);
+  if (e == cudaSuccess) s->adam_step += fused_out.steps;
+  if (hist_d && e == cudaSuccess && !fused_out.status) {
     e = cudaMemcpy(loss_hist_h, hist_d, sizeof(float) * (size_t)steps, cudaMemcpyDeviceToHost);
     for (int it = 0; it < steps; ++it) loss_hist_h[it] /= (float)batch;
   }
@@ -1576,6 +1587,7 @@ int cem_surrogate_train(cem_surrogate_handle s, const float* x_d, const float* t
   cudaFree(Xall);
   cudaFree(hist_d);
   if (e != cudaSuccess) return fail(CEM_ERR_CUDA, std::string("cem_surrogate_train: ") + cudaGetErrorString(e));
+  if (fused_out.status) return train_expired(s, fused_out.status);
   return CEM_OK;
 }
 
