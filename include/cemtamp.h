@@ -455,7 +455,8 @@ int cem_surrogate_set_forward_path(cem_surrogate_handle s, int path);
  * pipeline wait runs out after 1 s with nothing in flight; the CTA then
  * frees its TMEM, writes NaN scores and sets status 1.  The fused training
  * step does the same in its first launch (status 2), or, with on = 2, in its
- * second (status 12); cem_surrogate_gradient and cem_surrogate_train then
+ * second (status 12), or, with on = 3, leaves out the arrival that says that
+ * all of the second's MMAs are done (status 14); cem_surrogate_gradient and cem_surrogate_train then
  * return CEM_ERR_TIMEOUT.  The context stays usable; switch it off (0) for
  * normal calls. */
 int cem_surrogate_test_expire_wait(cem_surrogate_handle s, int on);
@@ -493,7 +494,7 @@ int cem_surrogate_get_adam_state(cem_surrogate_handle s, float* m1_h, float* m2_
 /* Synchronises, writes and clears the status word of the tcgen05 kernels: 0,
  * or the code of an expired wait: forward 1 / 2 (the weight copy / the MMAs),
  * which also makes cem_solve_screened return CEM_ERR_TIMEOUT; fused training
- * step 1 to 9 (its first launch: rows) and 11 to 13 (its second: weights). */
+ * step 1 to 9 (its first launch: rows) and 11 to 14 (its second: weights). */
 int cem_surrogate_status(cem_surrogate_handle s, int* status_h);
 /* Full-batch gradient of mean((out - (t - mu)/sigma)^2) over M rows into
  * grad_h (num_params floats) and the loss into *loss_h.  Synchronous.

@@ -352,7 +352,7 @@ struct TrainArgs {
   float lr, b1, b2, eps, wd;
   int* step_d;
   long long* adam_t_d;
-  int expire_test;  // failure-detection test: whose copy to leave out, 1 rows, 2 weights
+  int expire_test;  // failure-detection test: what to leave out, 1 a copy of rows, 2 of weights, 3 weights' last arrival
 };
 bool train_supported(int in_dim, int width, int depth);
 size_t train_pack_bytes();

@@ -38,7 +38,9 @@
 // of the same rows, bias, GELU and GELU' in FP32 afterwards, every sum in the
 // same fixed order), so both train the same network bit for bit.
 //
-// Waits are bounded (1 s of global time); on expiry the CTA sets out->status,
+// Waits are bounded (the thread that issues copies and MMAs: 1 s of global
+// time a wait in rows, for all of a CTA's rounds together in weights; threads
+// that wait for it: 2 s); on expiry the CTA sets out->status,
 // waits (bounded) for its own copies and MMAs, frees its TMEM and returns.
 // From then on the launches of the call do nothing: rows and weights give up
 // at their first look at the status and update writes nothing, so the
@@ -114,9 +116,11 @@ __device__ __forceinline__ uint64_t global_ns() {
   return t;
 }
 // wait for the phase with parity `phase`; false once the limit has passed
-// without it, or another thread of the CTA has given up (*fail)
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t phase, volatile int* fail, uint64_t limit = kWaitLimitNs) {
-  uint64_t t0 = 0;
+// without it, or another thread of the CTA has given up (*fail).  The limit
+// runs from `since`, set (from 0) by the first wait that has to poll: waits
+// that share it have one limit together.
+__device__ __forceinline__ bool mbar_wait_since(uint32_t bar, uint32_t phase, volatile int* fail, uint64_t& since,
+                                                uint64_t limit = kWaitLimitNs) {
   for (;;) {
     uint32_t done;
     asm volatile(
@@ -127,9 +131,13 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t phase, volatile
     if (done) return true;
     if (fail && *fail) return false;
     const uint64_t t = global_ns();
-    if (t0 == 0) t0 = t;
-    else if (t - t0 > limit) return false;
+    if (since == 0) since = t;
+    else if (t - since > limit) return false;
   }
+}
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t phase, volatile int* fail, uint64_t limit = kWaitLimitNs) {
+  uint64_t since = 0;
+  return mbar_wait_since(bar, phase, fail, since, limit);
 }
 // one thread: `bytes` (a multiple of 16) from global to shared in pieces of at
 // most 16 KB, counted on `bar`, on which the caller has announced them
@@ -571,6 +579,7 @@ __global__ void __launch_bounds__(BTHREADS, 2) train_weights_kernel(const TrainA
     const uint32_t idesc = make_idesc(N, 0, 0), idesc1 = make_idesc(16, 0, 0);
     int issued = 0;  // rounds whose copies were issued
     int used = 0;    // rounds whose MMAs were issued
+    uint64_t since = 0;  // one limit for all rounds, however many
     auto first = [&](int i) { return max(rbeg, (tile0 + i) * R); };
     auto rows_of = [&](int i) { return min(rend, (tile0 + i + 1) * R) - first(i); };
     auto copy = [&](int i) {
@@ -590,7 +599,7 @@ __global__ void __launch_bounds__(BTHREADS, 2) train_weights_kernel(const TrainA
     if (step_status(a)) s_fail = 10;
     for (; used < nsub && !s_fail; ++used) {
       const int sl = used % BSTAGES, rows = rows_of(used);
-      if (!mbar_wait(fullb + 8 * sl, (uint32_t)(used / BSTAGES) & 1u, &s_fail)) { s_fail = 12; break; }
+      if (!mbar_wait_since(fullb + 8 * sl, (uint32_t)(used / BSTAGES) & 1u, &s_fail, since)) { s_fail = 12; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t st = base + (uint32_t)sl * kStage, kb = group_bytes(N);
       const uint64_t da = make_desc(st, 2048u, 128u), db = make_desc(st + kStageA, kb, 128u);
@@ -605,22 +614,27 @@ __global__ void __launch_bounds__(BTHREADS, 2) train_weights_kernel(const TrainA
       if (issued < nsub) {  // the next copies take the stage of the round before, once its MMAs have read it
         const int prev = issued - BSTAGES;
         if (prev < used) {
-          if (!mbar_wait(freeb + 8 * (prev % BSTAGES), (uint32_t)(prev / BSTAGES) & 1u, &s_fail)) { ++used; s_fail = 11; break; }
+          if (!mbar_wait_since(freeb + 8 * (prev % BSTAGES), (uint32_t)(prev / BSTAGES) & 1u, &s_fail, since)) { ++used; s_fail = 11; break; }
           copy(issued);
           ++issued;
         }
       }
     }
+    if (!s_fail) {
+      // (the failure-detection test leaves the arrival out)
+      if (a.expire_test != 3) commit(doneb);
+      // waited for here too: this thread's limit is what the others go by
+      if (!mbar_wait_since(doneb, 0u, &s_fail, since)) s_fail = 14;
+    }
     if (s_fail) {  // (bounded) what is in flight lands first
-      for (int i = used; i < issued; ++i) mbar_wait(fullb + 8 * (i % BSTAGES), (uint32_t)(i / BSTAGES) & 1u, nullptr);
-      if (used > 0) mbar_wait(freeb + 8 * ((used - 1) % BSTAGES), (uint32_t)((used - 1) / BSTAGES) & 1u, nullptr);
-    } else {
-      commit(doneb);
+      since = 0;
+      for (int i = used; i < issued; ++i) mbar_wait_since(fullb + 8 * (i % BSTAGES), (uint32_t)(i / BSTAGES) & 1u, nullptr, since);
+      if (used > 0) mbar_wait_since(freeb + 8 * ((used - 1) % BSTAGES), (uint32_t)((used - 1) / BSTAGES) & 1u, nullptr, since);
     }
   }
   __syncwarp();
   bool ok = true;
-  if (!mbar_wait(doneb, 0u, &s_fail, 4 * kWaitLimitNs * (uint64_t)nsub)) {
+  if (!mbar_wait(doneb, 0u, &s_fail, 2 * kWaitLimitNs)) {
     ok = false;
     if (!s_fail) s_fail = 13;
   }

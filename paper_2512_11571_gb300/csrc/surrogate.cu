@@ -1394,7 +1394,7 @@ int cem_surrogate_set_forward_path(cem_surrogate_handle s, int path) {
 
 int cem_surrogate_test_expire_wait(cem_surrogate_handle s, int on) {
   if (!s) return fail(CEM_ERR_INVALID_ARG, "null handle");
-  s->expire_test = on == 2 ? 2 : on ? 1 : 0;
+  s->expire_test = on == 2 || on == 3 ? on : on ? 1 : 0;
   return CEM_OK;
 }
 

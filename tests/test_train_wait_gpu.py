@@ -1,5 +1,5 @@
 """The fused training step's bounded waits: one that runs out (the test hook
-leaves a copy out, so the wait has nothing in flight) ends the call with
+leaves a copy or an arrival out, so the wait has nothing in flight) ends the call with
 CEM_ERR_TIMEOUT and its code, changes no parameter, moment or counter, and the
 next call on the same handle is the one that never failed."""
 import time
@@ -10,8 +10,8 @@ import pytest
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-# hook value -> status: the first weights of the rows launch, the first operands of the weights launch
-WAITS = [(1, 2), (2, 12)]
+# hook value -> status: the first weights of the rows launch, the first operands of the weights launch, its last MMAs
+WAITS = [(1, 2), (2, 12), (3, 14)]
 
 
 @pytest.fixture(scope="module")
@@ -80,3 +80,12 @@ def test_expired_gradient_wait(P, hook, code):
         P.cem_surrogate_test_expire_wait(S.h, 0)
         g2, loss2 = S.gradient(x, t)
         assert S.status() == 0 and np.array_equal(g, g2) and loss == loss2
+
+
+def test_the_limit_does_not_grow_with_the_rows(P):
+    """64 rounds a CTA have one limit together (and CTAs that start later leave at once)."""
+    x, t = rows(32 * 64 * 64, 4)
+    with P.Surrogate(256, 4, seed=2) as S:
+        P.cem_surrogate_test_expire_wait(S.h, 3)
+        timed_out(P, lambda: S.gradient(x, t))
+        assert S.status() == 14
