@@ -42,9 +42,10 @@
 // time a wait in rows, for all of a CTA's rounds together in weights; threads
 // that wait for it: 2 s); on expiry the CTA sets out->status,
 // waits (bounded) for its own copies and MMAs, frees its TMEM and returns.
-// From then on the launches of the call do nothing: rows and weights give up
-// at their first look at the status and update writes nothing, so the
-// parameters are those after the last whole step.
+// From then on the launches of the call change nothing: rows and weights, which
+// look at the status beside their first loads, wait for nothing that is not
+// there yet, and update writes nothing, so the parameters are those after the
+// last whole step.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -184,8 +185,8 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
 // wrote or read only after grid_wait, which returns when that one is complete.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-// The status is looked at while the first copies are under way (it costs no
-// time there) and set by the first that gives up.
+// The status is looked at by a thread that does not issue (by the issuing one,
+// a look cost 0.2 us a launch) and set by the first that gives up.
 __device__ __forceinline__ int step_status(const TrainArgs& a) { return *(volatile int*)&a.out->status; }
 __device__ __forceinline__ void step_failed(const TrainArgs& a, int code) { atomicCAS(&a.out->status, 0, code); }
 __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
@@ -268,7 +269,6 @@ __global__ void __launch_bounds__(THREADS, 1) train_rows_kernel(const TrainArgs 
       };
       // (the failure-detection test leaves the first weights' barrier without its arrival)
       if (a.expire_test != 1) load_half(0, weight_base(0), kW0Bytes);
-      if (step_status(a)) fail = 10;
       for (int l = 0; l < DEPTH && !fail; ++l) {
         const int K = l == 0 ? IN : W;
         // layer l's input is written and its accumulators are drained
@@ -343,6 +343,7 @@ __global__ void __launch_bounds__(THREADS, 1) train_rows_kernel(const TrainArgs 
     for (int l = 0; l < DEPTH; ++l)
       for (int i = tid; i < W; i += ETHREADS) sbias[l * W + i] = a.bias[l][i];
     for (int i = tid; i < W; i += ETHREADS) swout[i] = __bfloat162float(a.w_out[i]);
+    const int status = tid == 0 ? step_status(a) : 0;
     // the minibatch rows (drawn with replacement, or the caller's in order),
     // rounded to BF16 into the input image
     {
@@ -362,6 +363,7 @@ __global__ void __launch_bounds__(THREADS, 1) train_rows_kernel(const TrainArgs 
         for (int q = 0; q < 8; ++q) *reinterpret_cast<bf16*>(sm + SM_X + image_off(r, fb * 8 + q, IN)) = __float2bfloat16_rn(v[q]);
       }
     }
+    if (status) s_fail = 10;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("bar.sync 1, %0;" ::"n"(ETHREADS));  // biases staged
     if (lane == 0) mbar_arrive(opb);
@@ -573,6 +575,7 @@ __global__ void __launch_bounds__(BTHREADS, 2) train_weights_kernel(const TrainA
   const uint32_t tmem = *tmem_slot;
   grid_next();
   grid_wait();
+  if (tid == 32 && step_status(a)) s_fail = 10;
   // rounds: the parts of the chunk in each tile (chunks are multiples of 32 rows)
   const int tile0 = rbeg / R, nsub = (rend - 1) / R - tile0 + 1;
   if (tid == 0) {
@@ -596,8 +599,7 @@ __global__ void __launch_bounds__(BTHREADS, 2) train_weights_kernel(const TrainA
     };
     // (the failure-detection test leaves the first copies out)
     for (; issued < nsub && issued < BSTAGES && a.expire_test != 2; ++issued) copy(issued);
-    if (step_status(a)) s_fail = 10;
-    for (; used < nsub && !s_fail; ++used) {
+    for (; used < nsub; ++used) {
       const int sl = used % BSTAGES, rows = rows_of(used);
       if (!mbar_wait_since(fullb + 8 * sl, (uint32_t)(used / BSTAGES) & 1u, &s_fail, since)) { s_fail = 12; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -690,7 +692,8 @@ __global__ void __launch_bounds__(CTHREADS) train_update_kernel(const TrainArgs 
     s_c[0] = 1.0f - powf(a.b1, t);
     s_c[1] = 1.0f - powf(a.b2, t);
   }
-  const bool failed = step_status(a) != 0;  // (set by earlier launches only: the same in every thread)
+  // set by earlier launches only: the same in every thread (looked at once the sums are there: the load rides along)
+  const int failed = a.out->status;
   if (b >= kUpdate4) __syncthreads();
   if (b >= kUpdate4 && failed) return;
   auto apply = [&](int i, float g, int decay) -> float {  // returns the new parameter
@@ -787,8 +790,9 @@ __global__ void __launch_bounds__(CTHREADS) train_update_kernel(const TrainArgs 
       } else {
         a.out->loss = red[0];
         if (step) {
-          a.out->steps += 1;
-          if (a.hist) a.hist[*a.step_d - 1] = red[0];
+          const int k = *a.step_d;  // (counted by this step's weight launch)
+          a.out->steps = k;
+          if (a.hist) a.hist[k - 1] = red[0];
         }
       }
     }

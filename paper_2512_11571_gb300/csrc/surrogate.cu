@@ -1575,9 +1575,10 @@ int cem_surrogate_train(cem_surrogate_handle s, const float* x_d, const float* t
     for (; done < steps && e == cudaSuccess; ++done) e = exec ? cudaGraphLaunch(exec, st) : enqueue_step();
     if (exec) cudaGraphExecDestroy(exec);
   }
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   TrainOut fused_out{0.0f, 0, steps};
-  if (fused && steps > 0 && e == cudaSuccess) e = cudaMemcpy(&fused_out, ta.out, sizeof(fused_out), cudaMemcpyDeviceToHost);
+  if (fused && steps > 0 && e == cudaSuccess)
+    e = cudaMemcpyAsync(&fused_out, ta.out, sizeof(fused_out), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e == cudaSuccess) s->adam_step += fused_out.steps;
   if (hist_d && e == cudaSuccess && !fused_out.status) {
     e = cudaMemcpy(loss_hist_h, hist_d, sizeof(float) * (size_t)steps, cudaMemcpyDeviceToHost);
