@@ -808,7 +808,7 @@ struct cem_surrogate_ctx {
   float* loss_d = nullptr;
   float* splitk = nullptr;   // split-K partials of the weight gradients
   float* colpart = nullptr;  // row-chunk partials of the bias gradients
-  // fused training step (csrc/mlp_train.cu): its workspace, one block
+  // fused training step (csrc/mlp_train.cu): its workspace, one block beside the row workspace
   uint8_t* train_work = nullptr;
   size_t train_bytes = 0;
   // screening workspace
@@ -832,6 +832,14 @@ struct cem_surrogate_ctx {
 
 namespace {
 
+// the fused training step's block (nothing of it is used between calls)
+void sur_free_train(cem_surrogate_ctx* s) {
+  cudaFree(s->train_work);
+  s->train_work = nullptr;
+  s->train_bytes = 0;
+}
+
+// the row workspace (the layer-by-layer paths, screening)
 void sur_free_work(cem_surrogate_ctx* s) {
   cudaFree(s->xin);
   for (auto* a : s->act) cudaFree(a);
@@ -847,9 +855,6 @@ void sur_free_work(cem_surrogate_ctx* s) {
   cudaFree(s->loss_d);
   cudaFree(s->splitk);
   cudaFree(s->colpart);
-  cudaFree(s->train_work);
-  s->train_work = nullptr;
-  s->train_bytes = 0;
   s->splitk = nullptr;
   s->colpart = nullptr;
   s->xin = nullptr;
@@ -884,6 +889,10 @@ int ensure_rows(cem_surrogate_ctx* s, int M) {
   if (e != cudaSuccess) {
     cudaGetLastError();
     sur_free_work(s);
+    if (s->train_work) {  // its place may be what is missing
+      sur_free_train(s);
+      return ensure_rows(s, M);
+    }
     return fail(CEM_ERR_NO_MEMORY, "surrogate workspace allocation failed");
   }
   s->cap_M = M;
@@ -965,9 +974,7 @@ int train_args(cem_surrogate_ctx* s, const float* x_d, const float* t_d, int bat
   const size_t bpart = take(sizeof(float) * W * kTrainDepth * a.chunks), cpart = take(sizeof(float) * W * a.tiles);
   const size_t lpart = take(sizeof(float) * (((size_t)batch + 255) / 256)), out_at = take(sizeof(TrainOut));
   if (o > s->train_bytes || !s->train_work) {
-    cudaFree(s->train_work);
-    s->train_work = nullptr;
-    s->train_bytes = 0;
+    sur_free_train(s);
     if (dev_malloc(&s->train_work, o) != cudaSuccess) {
       cudaGetLastError();
       s->train_work = nullptr;
@@ -1337,6 +1344,7 @@ int cem_surrogate_destroy(cem_surrogate_handle s) {
   if (!s) return CEM_OK;
   cudaDeviceSynchronize();
   sur_free_work(s);
+  sur_free_train(s);
   void* ptrs[] = {s->p, s->pb, s->g, s->m1, s->m2, s->norm,
                   s->pool_theta, s->pool_x, s->pool_score, s->keep_idx, s->tc_pack, s->tc_status,
                   s->step_d, s->adam_t_d, s->stat_part};
