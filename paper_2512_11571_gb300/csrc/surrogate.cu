@@ -1812,6 +1812,7 @@ int solve_screened(cem_handle h, cem_surrogate_handle s, const float* scene16_h,
       SUR_CUDA(cudaStreamSynchronize(st));
       rc = cem_surrogate_train(s, rb.x, rb.t, filled, ft->batch < filled ? ft->batch : filled, ft->steps, ft->lr,
                                ft->weight_decay, ft->seed + (uint64_t)j, 0, nullptr);
+      if (rc == CEM_ERR_TIMEOUT) cudaMemset(s->tc_status, 0, sizeof(int));  // reported here, as below
       if (rc != CEM_OK) return rc;
     }
   }

@@ -7,6 +7,8 @@ import time
 import numpy as np
 import pytest
 
+import workload
+
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
@@ -89,3 +91,21 @@ def test_the_limit_does_not_grow_with_the_rows(P):
         P.cem_surrogate_test_expire_wait(S.h, 3)
         timed_out(P, lambda: S.gradient(x, t))
         assert S.status() == 14
+
+
+def test_fine_tuning_reports_it_once(P):
+    """The screened loop reports an expired wait of its fine-tuning and clears
+    the word, as it does for its scoring: the next run is not held to it."""
+    sc, sk, _ = workload.config(2, seed=1, T=200)
+    f16 = workload.scene_features(sc)
+    run = dict(seed=1, N=128, K=16, iters=2, n_pool=256)
+    with P.Scene(sc, sk) as Sc, P.Surrogate(256, 4, seed=2) as S:
+        want = Sc.solve_screened(S, f16, **run)
+        P.cem_surrogate_test_expire_wait(S.h, 2)
+        with pytest.raises(P.CemError) as err:
+            Sc.solve_screened(S, f16, finetune=dict(every=1, steps=2, batch=64, capacity=1280), **run)
+        assert err.value.code == -3 and "training" in str(err.value)
+        P.cem_surrogate_test_expire_wait(S.h, 0)
+        got = Sc.solve_screened(S, f16, **run)
+        assert S.status() == 0
+    assert got["best_J"] == want["best_J"] and np.array_equal(got["mean"], want["mean"])
