@@ -281,7 +281,9 @@ int cem_base_path(cem_handle h, float sx, float sy, float gx, float gy, float* x
  * Synchronises the device, writes the first recorded code to *code_out (0:
  * none; 1 dispatch-order entry, 2 rollout-order entry, 3 rollout-order
  * position, 4 order bin, 5 dispatch-order position, 6 geometry index,
- * 7 parameter index, 8 elite index, 9 screened row index) and, if reset,
+ * 7 parameter index, 8 elite index, 9 screened row index, 10 / 11 a contact
+ * query of the base / the object left out that would have found something,
+ * 12 selection bin, 13 kept candidate, 14 drawn training row) and, if reset,
  * clears the record.  A release build writes 0 and returns
  * CEM_ERR_UNSUPPORTED. */
 int cem_debug_status(int* code_out, int reset);

@@ -967,13 +967,14 @@ int cem_debug_status(int* code_out, int reset) {
   if (!code_out) return fail(CEM_ERR_INVALID_ARG, "cem_debug_status: code_out is NULL");
   *code_out = 0;
 #ifdef CEM_DEBUG
-  int c[3] = {0, 0, 0};  // rollout.cu (rollouts, orders), refit.cu, surrogate.cu (screening)
+  int c[4] = {0, 0, 0, 0};  // rollout.cu (rollouts, orders), refit.cu, surrogate.cu (screening), mlp_train.cu
   cudaError_t e = cudaDeviceSynchronize();
   if (e == cudaSuccess) e = debug_status_rollout(&c[0], reset != 0);
   if (e == cudaSuccess) e = debug_status_refit(&c[1], reset != 0);
   if (e == cudaSuccess) e = debug_status_surrogate(&c[2], reset != 0);
+  if (e == cudaSuccess) e = debug_status_train(&c[3], reset != 0);
   if (e != cudaSuccess) return cuda_fail(e, "cem_debug_status");
-  *code_out = c[0] ? c[0] : c[1] ? c[1] : c[2];
+  *code_out = c[0] ? c[0] : c[1] ? c[1] : c[2] ? c[2] : c[3];
   return CEM_OK;
 #else
   (void)reset;

@@ -200,7 +200,7 @@ __device__ __forceinline__ int train_row(const TrainArgs& a, int i, uint32_t ste
   if (a.draw_from == 0) return i;
   uint32_t r[4];
   philox4x32_10((uint32_t)i, step, 0x5AFEu, 0u, (uint32_t)a.seed, (uint32_t)(a.seed >> 32), r);
-  return (int)(((uint64_t)r[0] * (uint64_t)a.draw_from) >> 32);
+  return CEM_DIDX((int)(((uint64_t)r[0] * (uint64_t)a.draw_from) >> 32), a.draw_from, 14);
 }
 
 // ------------------------------------------------------------------- rows
@@ -809,6 +809,10 @@ __global__ void train_pack_kernel(const bf16* __restrict__ pb, const TrainArgs a
 }
 
 }  // namespace
+
+#ifdef CEM_DEBUG
+CEM_DEBUG_STATUS_ACCESSOR(debug_status_train)
+#endif
 
 bool train_supported(int in_dim, int width, int depth) { return in_dim == IN && width == W && depth == DEPTH; }
 

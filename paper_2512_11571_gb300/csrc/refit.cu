@@ -88,7 +88,7 @@ __device__ __forceinline__ Cut block_select(SelectShared& sh, Each each, uint32_
   for (int p = 0; p < kSelPasses; ++p) {
     const int bits = 32 - __clz(hi - lo), shift = bits > 11 ? bits - 11 : 0;
     each([&](uint32_t key) {
-      if (key != kNoKey && key >= lo && key <= hi) atomicAdd(&sh.hist[p][(key - lo) >> shift], 1u);
+      if (key != kNoKey && key >= lo && key <= hi) atomicAdd(&sh.hist[p][CEM_DIDX((key - lo) >> shift, kSelBins, 12)], 1u);
     });
     __syncthreads();
     const uint32_t a = sh.hist[p][2 * tid], b = sh.hist[p][2 * tid + 1];
@@ -315,7 +315,7 @@ __device__ __forceinline__ void refit_body(const RefitArgs& a) {
       sort_keys(keys, P);
     }
     if (a.elite_idx)
-      for (int e = tid; e < keff; e += RT) a.elite_idx[e] = (int)(keys[e] & 0xFFFFF);
+      for (int e = tid; e < keff; e += RT) a.elite_idx[e] = CEM_DIDX((int)(keys[e] & 0xFFFFF), a.N, 8);
     // elite e's parameter row (read through L2; the keys stay in shared memory)
     auto eth = [&](int e, int d) -> float { return a.theta[(size_t)CEM_DIDX((int)(keys[e] & 0xFFFFF), a.N, 8) * D + d]; };
     // statistics in FP64: 4 threads per output, fixed reduction order

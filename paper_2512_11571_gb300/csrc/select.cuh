@@ -17,6 +17,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "internal.h"
+
 namespace cem {
 
 constexpr int kSelThreads = 1024;
@@ -117,7 +119,7 @@ __device__ __forceinline__ Cut cluster_select(cooperative_groups::cluster_group&
   for (int p = 0; p < kSelPasses; ++p) {
     const int bits = 32 - __clz(hi - lo), shift = bits > 11 ? bits - 11 : 0;
     each([&](bool valid, uint32_t key) {
-      if (valid && key >= lo && key <= hi) atomicAdd(&sh.hist[p][(key - lo) >> shift], 1u);
+      if (valid && key >= lo && key <= hi) atomicAdd(&sh.hist[p][CEM_DIDX((key - lo) >> shift, kSelBins, 12)], 1u);
     });
     if (nc > 1) cl.sync();
     else __syncthreads();

@@ -621,7 +621,7 @@ __global__ void __launch_bounds__(kSelThreads) topk_kernel(const float* __restri
     const uint32_t nt = ot + ties[j * 32 + w] + (uint32_t)__popc(bt & lt);
     if (lo || (eq && nt < take)) {
       const uint32_t pos = nb + min(nt, take);
-      if (pos < (uint32_t)keep) idx[pos] = first + j * kSelThreads + tid;
+      if (pos < (uint32_t)keep) idx[pos] = CEM_DIDX(first + j * kSelThreads + tid, N, 13);
     }
     ++j;
   });
