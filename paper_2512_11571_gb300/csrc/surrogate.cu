@@ -1505,10 +1505,12 @@ int cem_surrogate_train(cem_surrogate_handle s, const float* x_d, const float* t
   const bool fused = use_fused_train(s);
   // layer-by-layer path: the whole data set in BF16 once (the fused step rounds the rows it draws)
   bf16* Xall = nullptr;
-  float* hist_d = nullptr;  // per-step losses stay on the device until the end (no per-step sync)
+  // per-step losses stay on the device until the end (no per-step sync), and the fused step's report behind them
+  // (one copy for both; a copy of its own took 16 us)
+  float* hist_d = nullptr;
   cudaStream_t st = nullptr;
   if ((!fused && dev_malloc(&Xall, sizeof(bf16) * (size_t)M * s->in_dim) != cudaSuccess) ||
-      (loss_hist_h && steps > 0 && dev_malloc(&hist_d, sizeof(float) * (size_t)steps) != cudaSuccess)) {
+      (loss_hist_h && steps > 0 && dev_malloc(&hist_d, sizeof(float) * (size_t)steps + sizeof(TrainOut)) != cudaSuccess)) {
     cudaGetLastError();
     cudaFree(Xall);
     return fail(CEM_ERR_NO_MEMORY, "training set does not fit");
@@ -1556,6 +1558,7 @@ int cem_surrogate_train(cem_surrogate_handle s, const float* x_d, const float* t
     ta.draw_from = M;
     ta.seed = seed;
     ta.hist = hist_d;
+    if (hist_d) ta.out = reinterpret_cast<TrainOut*>(hist_d + steps);
     ta.lr = lr;
     ta.b1 = b1;
     ta.b2 = b2;
@@ -1583,15 +1586,20 @@ int cem_surrogate_train(cem_surrogate_handle s, const float* x_d, const float* t
     for (; done < steps && e == cudaSuccess; ++done) e = exec ? cudaGraphLaunch(exec, st) : enqueue_step();
     if (exec) cudaGraphExecDestroy(exec);
   }
-  TrainOut fused_out{0.0f, 0, steps};
-  if (fused && steps > 0 && e == cudaSuccess)
-    e = cudaMemcpyAsync(&fused_out, ta.out, sizeof(fused_out), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e == cudaSuccess) s->adam_step += fused_out.steps;
-  if (hist_d && e == cudaSuccess && !fused_out.status) {
-    e = cudaMemcpy(loss_hist_h, hist_d, sizeof(float) * (size_t)steps, cudaMemcpyDeviceToHost);
-    for (int it = 0; it < steps; ++it) loss_hist_h[it] /= (float)batch;
+  TrainOut fused_out{0.0f, 0, steps};
+  if (hist_d && e == cudaSuccess) {
+    std::vector<uint8_t> got(sizeof(float) * (size_t)steps + (fused ? sizeof(TrainOut) : 0));
+    e = cudaMemcpy(got.data(), hist_d, got.size(), cudaMemcpyDeviceToHost);
+    if (fused) std::memcpy(&fused_out, got.data() + sizeof(float) * (size_t)steps, sizeof(TrainOut));
+    if (e == cudaSuccess && !fused_out.status) {
+      std::memcpy(loss_hist_h, got.data(), sizeof(float) * (size_t)steps);
+      for (int it = 0; it < steps; ++it) loss_hist_h[it] /= (float)batch;
+    }
+  } else if (fused && steps > 0 && e == cudaSuccess) {
+    e = cudaMemcpy(&fused_out, ta.out, sizeof(fused_out), cudaMemcpyDeviceToHost);
   }
+  if (e == cudaSuccess) s->adam_step += fused_out.steps;
   cudaStreamDestroy(st);
   cudaFree(Xall);
   cudaFree(hist_d);
