@@ -465,23 +465,27 @@ int cem_surrogate_test_expire_wait(cem_surrogate_handle s, int on);
 /* The path inference takes now: 1 tiled GEMM, 2 tcgen05; -1 for NULL. */
 int cem_surrogate_forward_path(cem_surrogate_handle s);
 /* Dense layers of training (cem_surrogate_gradient, cem_surrogate_train)
- * and of the layer-by-layer inference forward: 0 automatic or 2 = the
- * tcgen05 GEMM (128 x 64 tiles, both operand majors read straight
- * by the tensor core, fused bias + GELU / GELU' / split-K epilogues; a layer
- * whose shape it does not take runs on the tiled kernel), 1 = the tiled
- * mma.sync GEMM.  Same products, FP32 accumulation order differs.  3 = an
- * FP32 debug path for cem_surrogate_gradient only: FP32 inputs, the FP32
- * master weights, FP32 activations and gradients, FP32 SIMT products summed
- * in ascending index order (no BF16 rounding anywhere; slow); training and
- * inference then take the automatic path.  Errors: CEM_ERR_INVALID_ARG for
- * another value.  A tcgen05 GEMM whose bounded wait expires sets status
- * 1 / 2 (read by cem_surrogate_status). */
+ * and of the layer-by-layer inference forward: 0 automatic or 2 = tcgen05:
+ * with width 256 and depth 4 training takes the fused step (three launches:
+ * rows forward and backward, weight gradients, update); other shapes, and the
+ * layer-by-layer forward, the tcgen05 GEMM (128 x 64 tiles, both operand
+ * majors read straight by the tensor core, fused bias + GELU / GELU' /
+ * split-K epilogues; a layer whose shape it does not take runs on the tiled
+ * kernel).  The two give the same bits.  1 = the tiled mma.sync GEMM: same
+ * products, FP32 accumulation order differs.  3 = an FP32 debug path for
+ * cem_surrogate_gradient only: FP32 inputs, the FP32 master weights, FP32
+ * activations and gradients, FP32 SIMT products summed in ascending index
+ * order (no BF16 rounding anywhere; slow); cem_surrogate_train then runs
+ * layer by layer on the tcgen05 GEMM whatever the shape, inference takes the
+ * automatic path.  Errors: CEM_ERR_INVALID_ARG for another value.  A tcgen05
+ * GEMM whose bounded wait expires sets status 1 / 2 (read by
+ * cem_surrogate_status); the fused step: see there. */
 int cem_surrogate_set_gemm_path(cem_surrogate_handle s, int path);
 /* The path training GEMMs take now: 1 tiled, 2 tcgen05, 3 the FP32 debug
  * gradient; -1 for NULL. */
 int cem_surrogate_gemm_path(cem_surrogate_handle s);
 /* One AdamW step of the training loop's optimiser with a given gradient
- * grad_h (num_params floats, host): the same kernel and state (FP32 master
+ * grad_h (num_params floats, host): the same arithmetic and state (FP32 master
  * weights, FP32 moments, the step counter that sets the bias correction,
  * beta 0.9 / 0.999, eps 1e-8, decoupled decay on weights only) as
  * cem_surrogate_train; the BF16 copy is refreshed.  set_params clears the

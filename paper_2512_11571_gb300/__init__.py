@@ -959,7 +959,8 @@ class Surrogate:
         return cem_surrogate_forward_path(self.h)
 
     def set_gemm_path(self, path):
-        """Training GEMMs: 0 automatic, 1 tiled mma.sync, 2 tcgen05, 3 the FP32 debug gradient."""
+        """Training: 0 automatic, 1 tiled mma.sync, 2 tcgen05 (the fused step where the shape allows),
+        3 the FP32 debug gradient (training then runs layer by layer on tcgen05)."""
         cem_surrogate_set_gemm_path(self.h, path)
 
     @property
@@ -983,7 +984,7 @@ class Surrogate:
         return cem_surrogate_get_adam_state(self.h)
 
     def status(self):
-        """Reads and clears the fused kernel's status word (0 = no wait expired)."""
+        """Reads and clears the tcgen05 kernels' status word (0 = no wait expired)."""
         return cem_surrogate_status(self.h)
 
     def train(self, x, t, batch=4096, steps=1000, lr=1e-3, weight_decay=1e-4, seed=0, normalize=True):

@@ -680,9 +680,10 @@ int set_last_error(int code, const std::string& msg) { return fail(code, msg); }
 int default_rollout_block(int N, int kind, int tpr, int envs) {
   // spread small batches over every SM scheduler: CTAs of 16 threads (each
   // half-warp its own warp, 4 schedulers per SM) up to one and a half warps a
-  // scheduler, larger CTAs after that, up to 128 threads.  Push, us with 16 /
-  // 32 / 64 threads: N = 4096 565 / 587 / 585, N = 8192 570 / 596 / 584, N =
-  // 16384 625 / 599 / 586; at N = 196,608 128 threads are 4 % faster than 256.
+  // scheduler, larger CTAs after that by the same measure, up to 128 threads.
+  // Push, us with 16 / 32 / 64 threads: N = 4096 565 / 587 / 585, N = 8192 570 /
+  // 596 / 584, N = 16384 625 / 599 / 586 (the rule takes 32 there; 64 is 2 %
+  // faster); at N = 196,608 128 threads are 4 % faster than 256.
   // The environments of a randomised sample are rollouts of their own here:
   // 1000 push samples in 8 environments 577 / 614 / 627, 1500 576 / 617 / 619.
   int sms = 152;

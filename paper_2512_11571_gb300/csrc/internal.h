@@ -63,7 +63,7 @@ struct DevScene {
   // mutual visibility (bit j of corner_vis[i]), built on the host
   int32_t base_ctrl, n_corners;
   float base_infl, wp_switch, pid_ki, pid_irad, pid_imax;
-  float sep_scale;  // 1 / the largest component of a slab normal beyond 1 (see take_budget)
+  float sep_scale;  // 1 / the largest component of a slab normal beyond 1 (rollout.cu, Reach::until)
   float corner[CEM_MAX_CORNERS][2];
   uint64_t corner_vis[CEM_MAX_CORNERS];
 };

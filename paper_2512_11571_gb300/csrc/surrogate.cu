@@ -565,7 +565,7 @@ __global__ void __launch_bounds__(kSelThreads) topk_kernel(const float* __restri
     __syncthreads();
     cut = cluster_select(cl, sh, each, (uint32_t)keep);
   }
-  // kept elements per (round, warp): below the cut in the low, ties in the high half of a pair of words
+  // kept elements per (round, warp): those below the cut and the ties, an array each
   uint32_t* below = rounds_sm;
   uint32_t* ties = rounds_sm + rounds * 32;
   int j = 0;
