@@ -80,7 +80,7 @@ def parse():
     ap.add_argument("--warps", type=int, default=4, help="warps per CTA of the persistent launch for --batch-only")
     ap.add_argument("--ctas", type=int, default=0, help="CTAs per SM of the persistent launch for --batch-only (0 = resident maximum)")
     ap.add_argument("--train-only", type=int, default=0,
-                    help="time this many surrogate training steps (batch 4096) on each GEMM path (profiling driver)")
+                    help="time this many surrogate training steps (batch 4096) on each training path (profiling driver)")
     return ap.parse_args()
 
 
@@ -563,7 +563,8 @@ def run_gb300(args):
                          "algorithmic_bytes": int(sum(p["N"] * (len(p["skel"]["lo"]) * 4 + 5) for p in probs)),
                          "peak_basis": f"{sms} SMs x 128 FP32 lanes x 2 x {mhz} MHz ({src} max SM clock)",
                          "kernel": "rollout_persistent_kernel",
-                         "flops_per_iteration": flops, "flops_basis": f"oracle op counts, {basis}",
+                         "flops_per_iteration": flops, "flops_basis": f"oracle op counts, {basis}, of all nominal N x T steps, also those "
+                                        "and the contact queries that the kernel leaves out",
                          "timing": "library stage events on the launching stream, every timed step"},
             "e2e": {"value": hd["e2e"], "unit": UNIT, "h2d_bytes_per_step": hd["e2e_bytes"],
                     "d2h_bytes_per_step": hd["e2e_bytes"], "api": "cem_batch_set_state -> cem_batch_iterate -> "
@@ -765,9 +766,9 @@ def run_batch_only(args):
 
 def run_train_only(args):
     """Times --train-only AdamW steps of the surrogate (48 -> 4 x 256 -> 1,
-    batch 4096 drawn from 65,536 stored rows) with the dense layers on the
-    tiled mma.sync GEMM and on the tcgen05 GEMM: 5 untimed steps, then the
-    timed ones (each cem_surrogate_train call ends with a device sync)."""
+    batch 4096 drawn from 65,536 stored rows) layer by layer on the tiled
+    mma.sync GEMM and on the tcgen05 GEMM, and by the fused tcgen05 step: 5
+    untimed steps, then the timed ones (each cem_surrogate_train call ends with a device sync)."""
     import numpy as np
     import torch
 
@@ -783,7 +784,7 @@ def run_train_only(args):
     # forward: 4 layers; backward: weight gradients of 4 layers, input gradients of 3
     gemm_flops = 2.0 * B * ((48 * 256 + 3 * 256 * 256) * 2 + 3 * 256 * 256)
     out = {"train_only": args.train_only, "batch": B, "gemm_gflop_per_step": gemm_flops / 1e9}
-    for path, name in ((1, "tiled_mma_sync"), (2, "tcgen05")):
+    for path, name in ((1, "tiled_mma_sync"), (3, "tcgen05_gemm"), (2, "fused_tcgen05")):
         with P.Surrogate(256, 4, seed=args.seed) as S:
             S.set_gemm_path(path)
             S.train(x, t, batch=B, steps=5, seed=1)
