@@ -566,6 +566,9 @@ int cem_batch_iterate_screened(cem_batch_handle h, int iters, void* stream) {
   if (!h) return fail(CEM_ERR_INVALID_ARG, "null handle");
   if (!h->sur) return fail(CEM_ERR_INVALID_ARG, "no surrogate set (cem_batch_set_screening)");
   if (iters < 0 || iters > 100000) return fail(CEM_ERR_UNSUPPORTED, "iters must be in 0..1e5");
+  // (the surrogate may have lost its rows since: another call that needed more of them found no memory)
+  const int rc = surrogate_reserve_pool(h->sur, h->n_pool, h->maxN, h->maxD);
+  if (rc != CEM_OK) return rc;
   cudaStream_t st = (cudaStream_t)stream;
   for (int j = 0; j < iters; ++j) {
     cudaError_t e = enqueue(h, st, true);
